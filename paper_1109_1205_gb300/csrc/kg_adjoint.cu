@@ -302,26 +302,6 @@ static int grad_pass(const kg_sector* sec, const double2* U, const double2* Wv, 
     return KG_OK;
 }
 
-// Lanczos space of every column's V_0 without the final combination (the
-// caller forms the vectors it needs at the times it needs).
-int build_space(Krylov& K, int reorth, cudaStream_t st) {
-    KG_TRY(launch_colnorm(K, st));
-    const bool ain = alpha_in_dots(K, reorth);
-    for (int j = 0; j < K.M; ++j) {
-        KG_TRY(launch_lanczos_hpsi(K, j, st, !ain));
-        if (reorth >= 1)
-            for (int k0 = 0; k0 <= j; k0 += kChunk)
-                KG_TRY(launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), false, st));
-        KG_TRY(launch_update(K, j, reorth, false, st));
-        if (reorth >= 2) {
-            for (int k0 = 0; k0 <= j; k0 += kChunk)
-                KG_TRY(launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), true, st));
-            KG_TRY(launch_update(K, j, reorth, true, st));
-        }
-    }
-    return KG_OK;
-}
-
 int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, int n_steps, const kg_opts* o,
                           int checkpoint, const double* dGgtr, const double* dGles, double* g_eps, double* g_hre,
                           double* g_him, double* g_U) {

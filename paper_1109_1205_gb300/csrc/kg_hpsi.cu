@@ -305,31 +305,55 @@ __global__ void __launch_bounds__(kThreads) k_hpsi(SecView S, const double2* __r
 // Lanczos step j for column b of a work-list launch:
 //   w = s_j H V_j - b_j s_{j-1} V_{j-1},   a_j = Re <s_j V_j, w>
 // (Eq. (recursion) with normalised v_k = s_k V_k).
+//
+// It starts by finishing what the update that made V_j left (resolve_norm),
+// and leaves the partial sums of a_j to the kernel after it: a reduction by
+// the reader costs one pass over a few hundred partials that every block does
+// at once, where a last block to arrive would add a fence, an atomic and a
+// serial tail to every launch.
 struct HpsiShared {
     double2 amp[kMaxL * kMaxL];
-    double sm[(kThreads / 32) * 2];
+    double sm[kThreads / 32];
     int smi[kThreads / 32];
-    double bs[2], red[2];
+    Partial pair[kThreads / 32];
     SecView S;
 };
 
 template <int MODE>
-__device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalars* cs, int j, int with_alpha,
-                                                  unsigned* cnt, const int4 it_, HpsiShared& sh) {
+__device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalars* cs, int j, const int4 it_,
+                                                  HpsiShared& sh) {
     const int b = it_.x, blk = it_.y, nblk = it_.z;
     const ColDesc D = desc[b];
     ColScalars* C = cs + b;
     SecView& S = sh.S;
     double2* amp = sh.amp;
-    double *sm = sh.sm, *bs = sh.bs, *red = sh.red;
-    int* smi = sh.smi;
-    if (j >= C->m_eff) return;
-    if (threadIdx.x == 0) S = *D.sec;
+    {
+        // the sector's view, word by word, and its amplitudes
+        static_assert(sizeof(SecView) % 8 == 0, "SecView is copied in 8-byte words");
+        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(D.sec);
+        for (int k = threadIdx.x; k < (int)(sizeof(SecView) / 8); k += blockDim.x)
+            reinterpret_cast<unsigned long long*>(&S)[k] = src[k];
+        if (MODE == 1 || MODE == 2) {
+            const int n = D.sec->L * D.sec->L;
+            const double2* ha = D.sec->hamp;
+            for (int k = threadIdx.x; k < n; k += blockDim.x) amp[k] = ha[k];
+        }
+    }
+    const bool writer = blk == 0 && threadIdx.x == 0;
+    NormHead H;
+    if (j > 0) {
+        H = resolve_norm(D, C, j, writer, sh.pair);
+    } else {  // the start vector's norm is k_colnorm's
+        H.m_eff = C->m_eff;
+        H.scale = C->scale[0];
+        H.emax = C->emax[0];
+        H.beta = 0.0;
+    }
+    if (j >= H.m_eff) return;
     __syncthreads();
-    stage_amplitudes(S, amp);
-    const double sj = C->scale[j];
-    const double cprev = (j > 0) ? C->beta[j] * C->scale[j - 1] : 0.0;
-    const int E = (MODE == 3) ? C->emax[j] : 0;
+    const double sj = H.scale;
+    const double cprev = (j > 0) ? H.beta * C->scale[j - 1] : 0.0;
+    const int E = (MODE == 3) ? H.emax : 0;
     const double hs = S.h0 * sj;
     // V_j in fixed point, written by the update that produced it (not V_0),
     // used when its exponent bound is tight enough
@@ -339,7 +363,7 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
     const double2* xp = D.V + (size_t)(j > 0 ? j - 1 : 0) * D.d;
     const int E0img = C->eimg[0];
     double2* w = D.W;
-    double acc[2] = {0.0, 0.0};
+    double acc = 0.0;
     int ew = 0;
     KG_FOR(idx) {
         int i_dn, i_up;
@@ -368,35 +392,19 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
         }
         w[idx] = r;
         if (j == 0 && D.I) D.I[idx] = fix_image(xv, E0img);  // image of V_0 for the exact dots
-        if (with_alpha) acc[0] = fma(xv.x, r.x, fma(xv.y, r.y, acc[0]));  // Re conj(x) r
+        acc = fma(xv.x, r.x, fma(xv.y, r.y, acc));  // Re conj(x) r
         ew = max(ew, max(exp_field(r.x), exp_field(r.y)));
     }
-    acc[0] *= sj;
-    ew = block_max_int(ew, smi);
-    block_sum<2>(acc, 1, sm, bs);
-    if (threadIdx.x == 0) bs[1] = (double)ew;
-    __syncthreads();
-    if (grid_finish(bs, 1, D.part, cnt + b, blk, nblk, red, 1)) {
-        if (threadIdx.x == 0) {
-            // without with_alpha, a_j = <v_j, w> comes from the exact dots
-            // (their coefficient of v_j), which the update adds to alpha[j]
-            const double a = with_alpha ? red[0] : 0.0;
-            C->alpha[j] = a;
-            C->ew = (int)red[1];
-            if (!isfinite(a)) {
-                C->status = KG_ENUMERIC;
-                C->m_eff = j + 1;
-            }
-        }
-    }
+    block_partial(sj * acc, ew, sh.sm, sh.smi, D.part_a + blk);
+    if (writer) C->n_alpha = nblk;
 }
 
 // One item per block (one-wave work lists, batches of any mix of sizes).
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 4) k_lanczos_hpsi(const ColDesc* desc, const int4* items, ColScalars* cs,
-                                                           int j, int with_alpha, unsigned* cnt) {
+                                                           int j) {
     __shared__ HpsiShared sh;
-    lanczos_hpsi_item<MODE>(desc, cs, j, with_alpha, cnt, items[blockIdx.x], sh);
+    lanczos_hpsi_item<MODE>(desc, cs, j, items[blockIdx.x], sh);
 }
 
 int launch_hpsi(kg_sector* s, const double2* x, double2* y, cudaStream_t st) {
@@ -453,7 +461,7 @@ int prepare_hpsi_lists(Krylov& K) {
     return KG_OK;
 }
 
-int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st, bool with_alpha) {
+int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st) {
     bool present[4] = {false, false, false, false};
     for (auto& D : K.hdesc) present[D.mode] = true;
     ProfScope ps("lanczos_hpsi", st);
@@ -469,10 +477,10 @@ int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st, bool with_alpha) {
         for (int g = 0; g < K.ngroups[mode]; ++g) {
             KG_TRY(work_list(K, kern, mode, &items, &n, g));
             switch (mode) {
-                case 3: k_lanczos_hpsi<3><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, with_alpha ? 1 : 0, K.cnt); break;
-                case 0: k_lanczos_hpsi<0><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, with_alpha ? 1 : 0, K.cnt); break;
-                case 1: k_lanczos_hpsi<1><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, with_alpha ? 1 : 0, K.cnt); break;
-                default: k_lanczos_hpsi<2><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, with_alpha ? 1 : 0, K.cnt); break;
+                case 3: k_lanczos_hpsi<3><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
+                case 0: k_lanczos_hpsi<0><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
+                case 1: k_lanczos_hpsi<1><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
+                default: k_lanczos_hpsi<2><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
             }
             KG_LAUNCHED();
         }

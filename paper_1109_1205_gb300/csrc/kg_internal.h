@@ -142,7 +142,17 @@ struct ColScalars {
     int ov_slot;                // overlap rows written so far
     int ew;                     // largest exponent field of the last H*psi output W
     int efix;                   // exponent of the fixed-point image Xf of the newest V_k
-    int pad;
+    // values a kernel leaves for its successors (see resolve_alpha, resolve_norm)
+    double araw;                // <v_j, w> of the current j, from the partial sums of H*psi
+    double abase, hre;          // a_j = abase + hre: the value before and the Gram-Schmidt correction
+    int n_alpha, n_norm;        // partial-sum rows written by H*psi and by the update
+    int eu;                     // exponent bound of the image of u in the exact dots
+};
+
+// One block's contribution to a column's sum: the value and a largest exponent.
+struct Partial {
+    double v;
+    long long e;
 };
 
 // One column of a Krylov batch.  Columns are independent vectors, each with
@@ -159,6 +169,9 @@ struct ColDesc {
     double2* W;             // [d] H v workspace
     double2* U;             // [d] W - a_j v_j, left by the Gram-Schmidt dots
     double* part;           // [nblk_max][kPart] partial sums of this column
+    Partial* part_a;        // [nblk_max] partial sums of a_j (H*psi), reduced by the next kernel
+    Partial* part_n;        // [nblk_max] partial sums of ||V_{j+1}||^2 (update), likewise
+    unsigned long long* gacc;  // [2][M + 1][4] exact dots: two 64-bit limbs of Re and Im each
     double2* out;           // where the combination writes (V_0 by default)
     const double2* ov;      // n_ov overlap vectors, stride ov_stride
     double2* ov_out;        // overlap rows [ov_rows][n_ov]
@@ -193,6 +206,8 @@ struct Krylov {
     longlong2* Xfbuf = nullptr;     // fixed-point H*psi inputs of exact-integer columns
     double2* Wbuf = nullptr;
     double* partbuf = nullptr;
+    Partial* pairbuf = nullptr;
+    unsigned long long* gaccbuf = nullptr;
     std::map<long long, std::pair<int4*, int>> lists;
     std::vector<int> group;         // H*psi launch group of each column (per mode)
     int ngroups[4] = {0, 0, 0, 0};  // groups per hop-sum mode
@@ -217,20 +232,18 @@ int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n,
 // y = H x (plain); exact-hop-sum sectors use the sector's own scratch.
 int launch_hpsi(kg_sector* s, const double2* x, double2* y, cudaStream_t st);
 // Lanczos H*psi: w = s_j H V_j - b_j s_{j-1} V_{j-1} for every column, with the
-// partial sums of a_j = <v_j, w> reduced on the device.
-// with_alpha = false leaves a_j to the exact Gram-Schmidt dots (alpha_in_dots).
-int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st, bool with_alpha = true);
-// True when the first Gram-Schmidt pass of level `reorth` runs the exact
-// integer dots, which then also give a_j = <v_j, w> (their coefficient of
-// v_j): H*psi skips its FP64 dot and the update subtracts a_j v_j.
-bool alpha_in_dots(const Krylov& K, int reorth);
+// partial sums of a_j = <v_j, w> left for the next kernel (resolve_alpha).
+int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st);
 // start of a step: beta0 = ||V_0||, scale[0], largest exponent, m_eff = M.
 int launch_colnorm(Krylov& K, cudaStream_t st);
 // Reorthogonalisation: h_k = <v_k, w - a_j v_j> (first pass) or
 // h_k = <v_k, V_{j+1}> (second pass) for k in [k0, k0 + nk).
 int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream_t st);
 // Lanczos update: V_{j+1} = w - a_j v_j - sum_k h_k v_k (or in place for the
-// second pass), then b_{j+1} = ||V_{j+1}||, scale, breakdown test.
+// second pass), with the partial sums of ||V_{j+1}||^2 left for the next
+// kernel (resolve_norm: b_{j+1}, scale, breakdown test).  launch_resolve does
+// that by itself, for a j + 1 that no H*psi follows.
+int launch_resolve(Krylov& K, int j, cudaStream_t st);
 // The Lanczos space (colnorm, then M iterations of H*psi, Gram-Schmidt and
 // update) of every column's V_0, without the combination step.
 int build_space(Krylov& K, int reorth, cudaStream_t st);
@@ -437,6 +450,32 @@ __device__ __forceinline__ int block_max_int(int v, int* sm) {
     return m;
 }
 
+// One block's partial sum and largest exponent, stored in *out.  The warps'
+// sums are added by one warp (a warp's FP64 instruction holds this GPU's FP64
+// pipe for many cycles, so eight serial adds by every thread would cost more
+// than the shuffles).  sm, smi: blockDim / 32 entries.
+__device__ __forceinline__ void block_partial(double v, int e, double* sm, int* smi, Partial* out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = warp_sum(v);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) {
+        sm[warp] = v;
+        smi[warp] = e;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < nw ? sm[lane] : 0.0;
+        e = lane < nw ? smi[lane] : 0;
+#pragma unroll
+        for (int o = kThreads / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) {
+            out->v = v;
+            out->e = e;
+        }
+    }
+}
+
 // Biased exponent field of an FP64 value (0 for zero).
 __device__ __forceinline__ int exp_field(double x) {
     return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
@@ -486,6 +525,94 @@ __device__ __forceinline__ int4 fix_image(double2 u, int E) {
 // costs one bit of the fixed-point sums' precision, which has P >= 4 bits to
 // spare over FP64), and converts on the fly otherwise.
 constexpr int kFixSlack = 4;
+
+// Sum of n partials and the largest of their exponents, in a fixed order, for
+// every thread of the block (every block of a launch gets the same bits).
+// sm: 2 * (blockDim / 32) doubles.
+__device__ __forceinline__ Partial sum_partials(const Partial* p, int n, Partial* sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int used = min(nw, (n + 31) >> 5);  // warps with anything to add
+    double s = 0.0;
+    int e = 0;
+    if (warp < used) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const Partial q = p[i];
+            s += q.v;
+            e = max(e, (int)q.e);
+        }
+        s = warp_sum(s);
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) {
+            sm[warp].v = s;
+            sm[warp].e = e;
+        }
+    }
+    __syncthreads();
+    if (used > 1) {
+        if (warp == 0) {
+            s = lane < used ? sm[lane].v : 0.0;
+            e = lane < used ? (int)sm[lane].e : 0;
+#pragma unroll
+            for (int o = kThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            e = __reduce_max_sync(0xffffffffu, e);
+            __syncwarp();
+            if (lane == 0) {
+                sm[0].v = s;
+                sm[0].e = e;
+            }
+        }
+        __syncthreads();
+    }
+    Partial r = sm[0];
+    return r;
+}
+
+// a_j = <v_j, w> and the largest exponent of w from the partial sums that
+// H*psi left (every block computes the same; `writer` also stores them).
+__device__ __forceinline__ double resolve_alpha(const ColDesc& D, ColScalars* C, bool writer, Partial* sm, int& ew) {
+    const Partial t = sum_partials(D.part_a, C->n_alpha, sm);
+    ew = (int)t.e;
+    if (writer) {
+        C->araw = t.v;
+        C->ew = ew;
+    }
+    return t.v;
+}
+
+// What the update that made V_j (j >= 1) leaves to the next kernel: b_j =
+// ||V_j||, s_j = 1/b_j, a_{j-1}, the largest exponent of V_j and the breakdown
+// test (the Krylov space is invariant when b_j is at rounding level relative
+// to |a_{j-1}| + b_{j-1}).  Every block computes the same values from the
+// partial sums; only `writer` stores them, so no block reads what another
+// may be writing (m_eff takes the same value before and after).
+struct NormHead {
+    double beta, scale;
+    int emax, m_eff;
+};
+
+__device__ __forceinline__ NormHead resolve_norm(const ColDesc& D, ColScalars* C, int j, bool writer, Partial* sm) {
+    NormHead h;
+    h.m_eff = C->m_eff;
+    h.beta = h.scale = 0.0;
+    h.emax = 0;
+    if (j - 1 >= h.m_eff) return h;  // the update did not run (block-uniform)
+    const double a = C->abase + C->hre, ref = fabs(a) + C->beta[j - 1];
+    const Partial t = sum_partials(D.part_n, C->n_norm, sm);
+    h.beta = sqrt(t.v);
+    h.scale = h.beta > 0.0 ? 1.0 / h.beta : 0.0;
+    h.emax = (int)t.e;
+    const bool bad = !isfinite(h.beta) || !isfinite(a);
+    if (bad || h.beta <= 1e-12 * fmax(ref, 1e-300)) h.m_eff = j;  // happy breakdown: K_j is invariant
+    if (writer) {
+        C->alpha[j - 1] = a;
+        C->beta[j] = h.beta;
+        C->scale[j] = h.scale;
+        C->emax[j] = h.emax;
+        C->m_eff = h.m_eff;
+        if (bad) C->status = KG_ENUMERIC;
+    }
+    return h;
+}
 
 // Deterministic reduction over the nblk blocks of one column (block `row`).
 // Each block stores its nv + nmax totals (bsum, in shared memory) into its

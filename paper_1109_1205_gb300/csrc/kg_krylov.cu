@@ -138,6 +138,8 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
     KG_TRY(need(cudaMalloc(&K.Wbuf, sizeof(double2) * 2 * nw), "work vector allocation"));
     if (nx) KG_TRY(need(cudaMalloc(&K.Xfbuf, sizeof(longlong2) * nx), "fixed-point image allocation"));
     KG_TRY(need(cudaMalloc(&K.partbuf, sizeof(double) * np), "partial-sum allocation"));
+    KG_TRY(need(cudaMalloc(&K.pairbuf, sizeof(Partial) * 2 * (np / kPart)), "partial-sum allocation"));
+    KG_TRY(need(cudaMalloc(&K.gaccbuf, sizeof(unsigned long long) * 8 * (size_t)K.B * (M + 1)), "dot allocation"));
     KG_TRY(need(cudaMalloc(&K.desc, sizeof(ColDesc) * K.B), "descriptor allocation"));
     KG_TRY(need(cudaMalloc(&K.secs, sizeof(SecView) * K.B), "sector view allocation"));
     KG_TRY(need(cudaMalloc(&K.cs, sizeof(ColScalars) * K.B), "scalar allocation"));
@@ -160,6 +162,9 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
         D.W = K.Wbuf + ow;
         D.U = K.Wbuf + nw + ow;
         D.part = K.partbuf + op;
+        D.part_a = K.pairbuf + 2 * (op / kPart);
+        D.part_n = D.part_a + D.nblk_max;
+        D.gacc = K.gaccbuf + 8 * (size_t)b * (M + 1);
         D.out = D.V;
         ov += (size_t)(M + 1) * D.d;
         ow += (size_t)D.d;
@@ -190,6 +195,8 @@ void krylov_free(Krylov& K) {
     cudaFree(K.Xfbuf);
     cudaFree(K.Wbuf);
     cudaFree(K.partbuf);
+    cudaFree(K.pairbuf);
+    cudaFree(K.gaccbuf);
     cudaFree(K.desc);
     cudaFree(K.secs);
     cudaFree(K.cs);
@@ -321,15 +328,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_reorth_dots(const ColDesc* desc
     constexpr int TG = kThreads / G;           // threads per group
     __shared__ double sm[(kThreads / 32) * 3 * KH];
     __shared__ double bs[3 * NK], red[3 * NK];
+    __shared__ Partial pair[kThreads / 32];
     KG_ITEM();
     if (j >= C->m_eff) return;
+    int ew;
+    const double araw = second ? 0.0 : resolve_alpha(D, C, blk == 0 && threadIdx.x == 0, pair, ew);
     const int d = D.d;
     const int grp = threadIdx.x / TG, t = threadIdx.x % TG;
     const int kb = grp * KH, kn = min(KH, NK - kb);
     const double2* Vb = D.V + (size_t)(k0 + kb) * d;
     const double2* w = second ? D.V + (size_t)(j + 1) * d : D.W;
     const double2* vj = D.V + (size_t)j * d;
-    const double aj = second ? 0.0 : C->alpha[j] * C->scale[j];
+    const double aj = second ? 0.0 : araw * C->scale[j];
     double acc[3 * KH];
 #pragma unroll
     for (int k = 0; k < 3 * KH; ++k) acc[k] = 0.0;
@@ -469,8 +479,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_reorth_dots_int(const ColDesc* 
     __shared__ double bs[2 * NK], red[2 * NK];
     __shared__ int eu_s;
     __shared__ int fresh_s[NK], ek_s[NK];
+    __shared__ Partial pair[kThreads / 32];
     KG_ITEM();
     if (j >= C->m_eff) return;
+    int ew;
+    const double araw = resolve_alpha(D, C, blk == 0 && threadIdx.x == 0, pair, ew);
     const int d = D.d;
     const int grp = threadIdx.x / TG, t = threadIdx.x % TG;
     const int kb = grp * KH, kn = min(KH, NK - kb);
@@ -478,22 +491,19 @@ __global__ void __launch_bounds__(kThreads, 3) k_reorth_dots_int(const ColDesc* 
     const double2* Vk = D.V + (size_t)(k0 + kb) * d;
     const double2* w = D.W;
     const double2* vj = D.V + (size_t)j * d;
-    const double aj = C->alpha[j] * C->scale[j];
-    // a_j = 0 here means a_j comes from these dots (u = W, which the update
-    // reads itself); otherwise the last chunk leaves u = W - a_j v_j in U
-    const bool sub = aj != 0.0;
-    const bool keep = sub && k0 + NK == j + 1;
+    const double aj = araw * C->scale[j];
+    // the last chunk leaves u = W - a_j v_j in U
+    const bool keep = k0 + NK == j + 1;
     if (threadIdx.x < NK) {
         ek_s[threadIdx.x] = C->emax[k0 + threadIdx.x];
         fresh_s[threadIdx.x] = C->eimg[k0 + threadIdx.x] - C->emax[k0 + threadIdx.x] > kFixSlack;
     }
     if (threadIdx.x == 0) {
         // |u_i| <= |W_i| + |a_j| |V_j[i]| < (1 + |a_j| 2^(E_j - E_w)) 2^(E_w - 1022), with a margin
-        const int Ew = C->ew;
-        const double r = (1.0 + fabs(aj) * ldexp(1.0, C->emax[j] - Ew)) * (1.0 + 1.0 / 1024.0);
+        const double r = (1.0 + fabs(aj) * ldexp(1.0, C->emax[j] - ew)) * (1.0 + 1.0 / 1024.0);
         int ex;
         const double fr = frexp(r, &ex);
-        eu_s = Ew + (fr == 0.5 ? ex - 1 : ex);
+        eu_s = ew + (fr == 0.5 ? ex - 1 : ex);
     }
     __syncthreads();
     const int Eu = eu_s;
@@ -514,11 +524,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_reorth_dots_int(const ColDesc* 
             const int e = threadIdx.x + r * kThreads, i = base + e;
             if (i < d) {
                 double2 u = w[i];
-                if (sub) {
-                    const double2 p = vj[i];
-                    u.x = fma(-aj, p.x, u.x);
-                    u.y = fma(-aj, p.y, u.y);
-                }
+                const double2 p = vj[i];
+                u.x = fma(-aj, p.x, u.x);
+                u.y = fma(-aj, p.y, u.y);
                 if (keep) D.U[i] = u;
                 const long long px = fix52(u.x, Eu), py = fix52(u.y, Eu);
                 up[e][0] = fix_hi(px);
@@ -616,13 +624,6 @@ static bool use_int_dots(const Krylov& K, bool second) {
     return true;
 }
 
-// a_j from the exact dots in the same pass as the Gram-Schmidt corrections
-// (classical Gram-Schmidt of w against v_0..v_j at once) loses
-// orthogonality over long Lanczos runs (a 120-step run past its exhausted
-// 100-state sector diverged); a_j is therefore always H*psi's FP64 dot, and
-// the exact dots correct it (u = w - a_j v_j first), as in the FP64 form.
-bool alpha_in_dots(const Krylov&, int) { return false; }
-
 int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream_t st) {
     ProfScope ps("reorth_dots", st);
     if (use_int_dots(K, second)) {
@@ -658,62 +659,98 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
 // than the FP64 pipe on this GPU.  Larger coefficients use FP64.
 constexpr double kSmallCoef = 1e-10;
 
+// Its first warp sorts the terms, one vector per lane: a serial pass by one
+// thread costs two dependent L2 reads and a few FP64 operations per vector in
+// every block.  With the sums reduced by the reader (resolve_norm) instead of
+// by the last block to arrive, a Lanczos iteration on a 300-state column at
+// M = 40 went from 53 to 38 us, on one 853,776-state column from 190 to 174 us.
 __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const int4* items, ColScalars* cs, int j,
-                                                     int level, int second, unsigned* cnt) {
+                                                     int level, int second) {
     // block-uniform term lists: FP32 terms (small coefficients), FP64 terms
     __shared__ double2 coef64[kMaxMgs + 1];
     __shared__ float2 coef32[kMaxMgs + 1];
     __shared__ int idx32[kMaxMgs + 1], idx64[kMaxMgs + 1];
     __shared__ int n32, n64, efix_s;
-    __shared__ double coefA;
-    __shared__ double sm[(kThreads / 32) * 2];
+    __shared__ double sm[kThreads / 32];
     __shared__ int smi[kThreads / 32];
-    __shared__ double bs[2], red[2];
+    __shared__ Partial pair[kThreads / 32];
     KG_ITEM();
     if (j >= C->m_eff) return;
+    const bool writer = blk == 0 && threadIdx.x == 0;
     const int d = D.d;
     double2* Vb = D.V;
     const int nk = (level >= 1 || second) ? j + 1 : 0;
-    // a first pass whose a_j came from the exact dots (alpha[j] still 0):
-    // Re h_j is a_j, subtracted here in FP64 (its tiny imaginary part joins
-    // the other Gram-Schmidt terms), from w itself
-    const bool ain = !second && level >= 1 && C->alpha[j] == 0.0;
-    if (threadIdx.x == 0) {
+    // a_j before the Gram-Schmidt correction: from the dots before a first
+    // pass, else (no Gram-Schmidt) straight from the partial sums of H*psi
+    int ew = 0;
+    double araw = 0.0;
+    if (second) {
+        ew = C->emax[j + 1];
+    } else if (nk) {
+        araw = C->araw;
+        ew = C->ew;
+    } else {
+        araw = resolve_alpha(D, C, writer, pair, ew);
+    }
+    const double aj = araw * C->scale[j];
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
         int a32 = 0, a64 = 0;
-        coefA = 0.0;
-        for (int k = 0; k < nk; ++k) {
-            const double s = C->scale[k];
-            double2 h = C->h[k];
-            if (ain && k == j) {
-                coefA = s * h.x;
-                h.x = 0.0;
+        // bound of the result's components, in units of 2^(ew - 1022) (below)
+        double r = 0.0;
+        for (int k0 = 0; k0 < nk; k0 += 32) {
+            const int k = k0 + lane;
+            double2 h = make_double2(0.0, 0.0), c = h;
+            if (k < nk) {
+                const double s = C->scale[k];
+                h = C->h[k];
+                c = make_double2(s * h.x, s * h.y);
+                r += (fabs(c.x) + fabs(c.y)) * ldexp(1.0, C->emax[k] - ew);
             }
-            const double2 c = make_double2(s * h.x, s * h.y);
-            if ((fabs(h.x) + fabs(h.y)) < kSmallCoef) {  // |h_k| for the unit vector v_k
-                coef32[a32] = make_float2((float)c.x, (float)c.y);
-                idx32[a32++] = k;
-            } else {
-                coef64[a64] = c;
-                idx64[a64++] = k;
+            const bool small = (fabs(h.x) + fabs(h.y)) < kSmallCoef;  // |h_k| for the unit vector v_k
+            const unsigned in = __ballot_sync(0xffffffffu, k < nk), ms = __ballot_sync(0xffffffffu, k < nk && small);
+            const unsigned before = (1u << lane) - 1u;
+            if (k < nk && small) {
+                const int q = a32 + __popc(ms & before);
+                coef32[q] = make_float2((float)c.x, (float)c.y);
+                idx32[q] = k;
+            } else if (k < nk) {
+                const int q = a64 + __popc(in & ~ms & before);
+                coef64[q] = c;
+                idx64[q] = k;
             }
+            a32 += __popc(ms);
+            a64 += __popc(in & ~ms);
         }
-        n32 = a32;
-        n64 = a64;
+        r = warp_sum(r);
+        if (lane == 0) {
+            n32 = a32;
+            n64 = a64;
+            // Every component of the result is below
+            //   2^(E_u - 1022) + |a_j| 2^(E_j - 1022) + sum_k (|Re c_k| + |Im c_k|) 2^(E_k - 1022)
+            // (E_u: largest exponent of W, or of V_{j+1} in a second pass),
+            // times a margin for the rounding of the FP64 and FP32 arithmetic.
+            r += 1.0;
+            if (!second) r += fabs(aj) * ldexp(1.0, C->emax[j] - ew);
+            r *= 1.0 + 1.0 / 1024.0;
+            int ex;
+            const double fr = frexp(r, &ex);  // r = fr * 2^ex, fr in [0.5, 1)
+            efix_s = ew + (fr == 0.5 ? ex - 1 : ex);
+        }
     }
     __syncthreads();
     const int m32 = n32, m64 = n64;
-    const double aj = C->alpha[j] * C->scale[j], cA = coefA;
     const double2* w = second ? Vb + (size_t)(j + 1) * d : D.W;
     const double2* vj = Vb + (size_t)j * d;
     double2* out = Vb + (size_t)(j + 1) * d;
     const float2* V32 = D.V32;
     double* S1 = D.S ? D.S + (size_t)(j + 1) * d : nullptr;
     float2* V32_1 = D.V32 ? D.V32 + (size_t)(j + 1) * d : nullptr;
-    double acc[1] = {0.0};
+    double acc = 0.0;
     int em = 0;
     // after a first-pass Gram-Schmidt (level >= 1) U holds W - a_j v_j
     const bool sub = !second && level < 1;
-    const double2* win = (!second && level >= 1 && !ain) ? D.U : w;
+    const double2* win = (!second && level >= 1) ? D.U : w;
     auto element = [&](int i) {
         double2 u = win[i];
         if (sub) {
@@ -767,11 +804,6 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
             u.x -= fma(c.x, v.x, -c.y * v.y);
             u.y -= fma(c.x, v.y, c.y * v.x);
         }
-        if (ain) {
-            const double2 p = vj[i];
-            u.x = fma(-cA, p.x, u.x);
-            u.y = fma(-cA, p.y, u.y);
-        }
         u.x -= f32_to_f64_int(cx);
         u.y -= f32_to_f64_int(cy);
         out[i] = u;
@@ -779,7 +811,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
             S1[i] = u.x + u.y;
             V32_1[i] = make_float2(f64_to_f32_trunc(u.x), f64_to_f32_trunc(u.y));
         }
-        acc[0] = fma(u.x, u.x, fma(u.y, u.y, acc[0]));
+        acc = fma(u.x, u.x, fma(u.y, u.y, acc));
         em = max(em, max(exp_field(u.x), exp_field(u.y)));
         return u;
     };
@@ -788,26 +820,8 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
         // Last pass of an exact-integer column: also write the fixed-point
         // image of V_{j+1} that the next H*psi reads, on the exponent efix;
         // with the exact dots, also its 52-bit image I_{j+1} on the same one.
-        // The vector's largest exponent is only known at the end of this
-        // kernel, so efix bounds it from the inputs: every component of the
-        // result is below
-        //   2^(E_u - 1022) + |a_j| 2^(E_j - 1022) + sum_k (|Re c_k| + |Im c_k|) 2^(E_k - 1022)
-        // (E_u: largest exponent of W, or of V_{j+1} in a second pass), times
-        // a margin for the rounding of the FP64 and FP32 arithmetic.
-        if (threadIdx.x == 0) {
-            const int Eu = second ? C->emax[j + 1] : C->ew;
-            double r = 1.0;
-            if (!second) r += (fabs(aj) + fabs(cA)) * ldexp(1.0, C->emax[j] - Eu);
-            for (int q = 0; q < m32; ++q)
-                r += (fabs((double)coef32[q].x) + fabs((double)coef32[q].y)) * ldexp(1.0, C->emax[idx32[q]] - Eu);
-            for (int q = 0; q < m64; ++q)
-                r += (fabs(coef64[q].x) + fabs(coef64[q].y)) * ldexp(1.0, C->emax[idx64[q]] - Eu);
-            r *= 1.0 + 1.0 / 1024.0;
-            int ex;
-            const double fr = frexp(r, &ex);  // r = fr * 2^ex, fr in [0.5, 1)
-            efix_s = Eu + (fr == 0.5 ? ex - 1 : ex);
-        }
-        __syncthreads();
+        // The vector's largest exponent is only known after this kernel, so
+        // efix bounds it from the inputs (the prologue).
         const int Ef = efix_s, P = D.fix_pre;
         int4* I1 = img ? D.I + (size_t)(j + 1) * d : nullptr;
         if (D.Xf && img) {
@@ -831,26 +845,26 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     } else {
         KG_FOR(i) element(i);
     }
-    em = block_max_int(em, smi);
-    block_sum<1>(acc, 1, sm, bs);
-    if (threadIdx.x == 0) bs[1] = (double)em;
-    __syncthreads();
-    if (grid_finish(bs, 1, D.part, cnt + b, blk, nblk, red, 1) && threadIdx.x == 0) {
-        C->emax[j + 1] = (int)red[1];
-        const double n = sqrt(red[0]);
-        double a = C->alpha[j];
-        if (nk) a += C->h[j].x;
-        C->alpha[j] = a;
-        C->beta[j + 1] = n;
-        C->scale[j + 1] = n > 0.0 ? 1.0 / n : 0.0;
-        const double ref = fabs(a) + C->beta[j];
-        if (!isfinite(n) || !isfinite(a)) {
-            C->status = KG_ENUMERIC;
-            C->m_eff = j + 1;
-        } else if (n <= 1e-12 * fmax(ref, 1e-300)) {
-            C->m_eff = j + 1;  // happy breakdown: K_{j+1} is invariant
-        }
+    block_partial(acc, em, sm, smi, D.part_n + blk);
+    if (writer) {
+        C->n_norm = nblk;
+        C->abase = second ? C->alpha[j] : araw;
+        C->hre = nk ? C->h[j].x : 0.0;
     }
+}
+
+// resolve_norm by itself, one block per column.
+__global__ void __launch_bounds__(kThreads) k_resolve(const ColDesc* desc, ColScalars* cs, int j) {
+    __shared__ Partial pair[kThreads / 32];
+    const ColDesc D = desc[blockIdx.x];
+    resolve_norm(D, cs + blockIdx.x, j, threadIdx.x == 0, pair);
+}
+
+int launch_resolve(Krylov& K, int j, cudaStream_t st) {
+    ProfScope ps("resolve", st);
+    k_resolve<<<K.B, kThreads, 0, st>>>(K.desc, K.cs, j);
+    KG_LAUNCHED();
+    return KG_OK;
 }
 
 int launch_update(Krylov& K, int j, int level, bool second, cudaStream_t st) {
@@ -858,7 +872,7 @@ int launch_update(Krylov& K, int j, int level, bool second, cudaStream_t st) {
     const int4* items;
     int n;
     KG_TRY(work_list(K, (const void*)k_update, -1, &items, &n));
-    k_update<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, level, second ? 1 : 0, K.cnt);
+    k_update<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, level, second ? 1 : 0);
     KG_LAUNCHED();
     return KG_OK;
 }
@@ -1210,28 +1224,41 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
     __shared__ double bs[2 * NOV + 2], red[2 * NOV + 2];
     KG_ITEM();
     const int m = C->m_eff;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {  // the first warp sorts the terms, one per lane
+        const int lane = threadIdx.x;
         double cmax = 0.0;
-        for (int k = 0; k < m; ++k) {
+        for (int k = lane; k < m; k += 32) {
             const double2 c = C->c[k];
             const double sk = C->scale[k];
             if (sk > 0.0) cmax = fmax(cmax, (fabs(c.x) + fabs(c.y)) / sk);
         }
+#pragma unroll
+        for (int o_ = 16; o_ > 0; o_ >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o_));
         int a64 = 0, a32 = 0;
-        for (int k = 0; k < m; ++k) {
-            const double2 c = C->c[k];
-            const double sk = C->scale[k];
-            if (D.V32 && sk > 0.0 && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk) {
-                coef32[a32] = make_float2((float)c.x, (float)c.y);
-                idx32[a32++] = k;
-            } else {
-                coef[a64] = c;
-                csum[a64] = c.x + c.y;
-                idx64[a64++] = k;
+        for (int k0 = 0; k0 < m; k0 += 32) {
+            const int k = k0 + lane;
+            const double2 c = k < m ? C->c[k] : make_double2(0.0, 0.0);
+            const double sk = k < m ? C->scale[k] : 0.0;
+            const bool small = D.V32 && sk > 0.0 && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
+            const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, k < m && small);
+            const unsigned before = (1u << lane) - 1u;
+            if (k < m && small) {
+                const int q = a32 + __popc(ms & before);
+                coef32[q] = make_float2((float)c.x, (float)c.y);
+                idx32[q] = k;
+            } else if (k < m) {
+                const int q = a64 + __popc(in & ~ms & before);
+                coef[q] = c;
+                csum[q] = c.x + c.y;
+                idx64[q] = k;
             }
+            a32 += __popc(ms);
+            a64 += __popc(in & ~ms);
         }
-        n64 = a64;
-        n32 = a32;
+        if (lane == 0) {
+            n64 = a64;
+            n32 = a32;
+        }
     }
     __syncthreads();
     const int m64 = n64, m32 = n32;
@@ -1420,21 +1447,27 @@ int prepare_step(Krylov& K, int reorth) {
     return KG_OK;
 }
 
-int enqueue_step(Krylov& K, int reorth, cudaStream_t st) {
+// Lanczos space of every column's V_0.
+int build_space(Krylov& K, int reorth, cudaStream_t st) {
     KG_TRY(launch_colnorm(K, st));
-    const bool ain = alpha_in_dots(K, reorth);
     for (int j = 0; j < K.M; ++j) {
-        KG_TRY(launch_lanczos_hpsi(K, j, st, !ain));
+        KG_TRY(launch_lanczos_hpsi(K, j, st));
         if (reorth >= 1)
             for (int k0 = 0; k0 <= j; k0 += kChunk)
                 KG_TRY(launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), false, st));
         KG_TRY(launch_update(K, j, reorth, false, st));
         if (reorth >= 2) {
+            KG_TRY(launch_resolve(K, j + 1, st));
             for (int k0 = 0; k0 <= j; k0 += kChunk)
                 KG_TRY(launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), true, st));
             KG_TRY(launch_update(K, j, reorth, true, st));
         }
     }
+    return launch_resolve(K, K.M, st);
+}
+
+int enqueue_step(Krylov& K, int reorth, cudaStream_t st) {
+    KG_TRY(build_space(K, reorth, st));
     KG_TRY(launch_tridiag(K, 0, st));
     KG_TRY(launch_combine(K, st));
     return KG_OK;
@@ -1471,18 +1504,7 @@ int ground_state(kg_sector* s, const kg_opts* o) {
     ColScalars h;
     bool converged = false;
     for (int r = 0; rc == KG_OK && r < o->max_restarts; ++r) {
-        if ((rc = launch_colnorm(K, st)) != KG_OK) break;
-        for (int j = 0; j < M && rc == KG_OK; ++j) {
-            rc = launch_lanczos_hpsi(K, j, st, !alpha_in_dots(K, 1));
-            for (int k0 = 0; rc == KG_OK && k0 <= j; k0 += kChunk)
-                rc = launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), false, st);
-            if (rc == KG_OK) rc = launch_update(K, j, std::max(1, o->reorth), false, st);
-            if (rc == KG_OK && o->reorth >= 2) {
-                for (int k0 = 0; rc == KG_OK && k0 <= j; k0 += kChunk)
-                    rc = launch_reorth_dots(K, j, k0, std::min(kChunk, j + 1 - k0), true, st);
-                if (rc == KG_OK) rc = launch_update(K, j, o->reorth, true, st);
-            }
-        }
+        rc = build_space(K, std::max(1, o->reorth), st);
         if (rc == KG_OK) rc = launch_tridiag(K, 1, st);
         if (rc == KG_OK) rc = launch_combine(K, st);
         if (rc != KG_OK) break;
