@@ -689,10 +689,7 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
         std::vector<ColScalars> h(NC);
         if (cudaMemcpy(h.data(), KB.cs, sizeof(ColScalars) * NC, cudaMemcpyDeviceToHost) != cudaSuccess) rc = KG_ECUDA;
         for (auto& c : h)
-            if (rc == KG_OK && c.status == KG_ENUMERIC) {
-                set_error("non-finite value in the adjoint sweep");
-                rc = KG_ENUMERIC;
-            }
+            if (rc == KG_OK) rc = column_rc(c.status, "the adjoint sweep");
     }
     if (NC > 0) {
         krylov_free(KF);

@@ -43,10 +43,7 @@ int propagate(kg_sector* s, double2* x, double dt, int n_steps, const kg_opts* o
         rc = cudaMemcpyAsync(&h, K.cs, sizeof(ColScalars), cudaMemcpyDeviceToHost, st) == cudaSuccess ? KG_OK : KG_ECUDA;
     if (rc == KG_OK)
         rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : cuda_fail(cudaGetLastError(), "propagate", __FILE__, __LINE__);
-    if (rc == KG_OK && h.status == KG_ENUMERIC) {
-        set_error("non-finite value during propagation");
-        rc = KG_ENUMERIC;
-    }
+    if (rc == KG_OK) rc = column_rc(h.status, "propagation");
     R.release();
     krylov_free(K);
     return rc;

@@ -409,14 +409,12 @@ static int green_eq_batch(kg_sector* const* sv, int n_inst, const int* orb, int 
     }
     if (rc == KG_OK) {
         for (auto& g : G) {
-            bool bad = false;
-            for (size_t a = 0; a < g.idx.size(); ++a) bad |= hcs[g.col0 + a].status == KG_ENUMERIC;
-            if (bad) {
-                if (status) status[g.inst] = KG_ENUMERIC;
-                if (n_inst == 1) {
-                    set_error("non-finite value during propagation");
-                    rc = KG_ENUMERIC;
-                }
+            int bad = KG_OK;
+            for (size_t a = 0; bad == KG_OK && a < g.idx.size(); ++a)
+                bad = column_rc(hcs[g.col0 + a].status, "propagation");
+            if (bad != KG_OK) {
+                if (status) status[g.inst] = bad;
+                if (n_inst == 1) rc = bad;
                 continue;
             }
             eq_assemble(g, hov, rows, dt, inst[g.inst]->E0, n_orb, G_gtr + per_inst * g.inst,
@@ -710,10 +708,7 @@ static int green_restarted(kg_sector* s, const int* orb, int n_orb, int n, int f
             for (int bcol = 0; bcol < na; ++bcol) {
                 const int b = g.col0 + bcol;
                 const ColScalars& c = hcs[b];
-                if (c.status == KG_ENUMERIC) {
-                    set_error("non-finite value in the restarted Lanczos run");
-                    return release(KG_ENUMERIC);
-                }
+                if ((rc = column_rc(c.status, "the restarted Lanczos run")) != KG_OK) return release(rc);
                 const int m = c.m_eff;
                 double2* cnext = hc.data() + (size_t)b * K.M;
                 for (int k = 0; k < K.M; ++k) cnext[k] = make_double2(0.0, 0.0);
@@ -930,10 +925,7 @@ int green_matsubara_steps(kg_sector* s, const int* orb, int n_orb, double mu, do
             const double shift = g.dagger ? s->E0 + mu : s->E0 - mu;
             for (int bcol = 0; bcol < na; ++bcol) {
                 const int b = g.col0 + bcol, m = hcs[b].m_eff;
-                if (hcs[b].status == KG_ENUMERIC) {
-                    set_error("non-finite value during the imaginary-time steps");
-                    return release(KG_ENUMERIC);
-                }
+                if ((rc = column_rc(hcs[b].status, "the imaginary-time steps")) != KG_OK) return release(rc);
                 double2* c = hc.data() + (size_t)b * K.M;
                 const int erc = imag_step_error(imag_step_coefficients(hcs[b], shift, dtau, K.M, c), dtau, K.M);
                 if (erc != KG_OK) return release(erc);
@@ -1022,11 +1014,7 @@ int imag_time_vectors(kg_sector* s, const int* orb, const std::vector<int>& idx,
              cudaStreamSynchronize(st) != cudaSuccess))
             rc = cuda_fail(cudaGetLastError(), "imaginary-time readback", __FILE__, __LINE__);
         for (int a = 0; rc == KG_OK && a < na; ++a) {
-            if (hcs[a].status == KG_ENUMERIC) {
-                set_error("non-finite value during the imaginary-time steps");
-                rc = KG_ENUMERIC;
-                break;
-            }
+            if ((rc = column_rc(hcs[a].status, "the imaginary-time steps")) != KG_OK) break;
             rc = imag_step_error(imag_step_coefficients(hcs[a], shift, dtau, K.M, hc.data() + (size_t)a * K.M), dtau,
                                  K.M);
         }
@@ -1254,10 +1242,7 @@ static int block_status_of(Krylov& K, const char* what) {
     std::vector<ColScalars> h(K.B);
     KG_CUDA(cudaMemcpy(h.data(), K.cs, sizeof(ColScalars) * K.B, cudaMemcpyDeviceToHost));
     for (auto& c : h)
-        if (c.status == KG_ENUMERIC) {
-            set_error("non-finite value during %s", what);
-            return KG_ENUMERIC;
-        }
+        KG_TRY(column_rc(c.status, what));
     return KG_OK;
 }
 

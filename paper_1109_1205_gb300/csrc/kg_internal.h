@@ -138,7 +138,7 @@ struct ColScalars {
     double rq, rnorm;           // Rayleigh quotient and residual of a Ritz vector
     double ovnorm;              // norm of the last combined vector
     int m_eff;                  // Krylov dimension reached (smaller after a breakdown)
-    int status;                 // KG_OK, KG_ENUMERIC or KG_ENOCONV
+    int status;                 // KG_OK, KG_ENUMERIC, KG_ENOCONV or KG_ETIMEOUT
     int ov_slot;                // overlap rows written so far
     int ew;                     // largest exponent field of the last H*psi output W
     int efix;                   // exponent of the fixed-point image Xf of the newest V_k
@@ -180,7 +180,7 @@ struct ColDesc {
     int d, n_ov, ov_rows, nblk_max;
     int mode;               // hop sums: 0 FP64 uniform, 1 real, 2 complex, 3 exact integer
     int Du, Dd, fix_pre;    // row length, row count, fixed-point pre-shift of the sector
-    int pad;
+    int M;                  // Krylov dimension of the workspace
 };
 
 // B columns of (possibly) different sectors.  Every streaming kernel runs over
@@ -226,7 +226,8 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
 size_t krylov_bytes(const std::vector<const kg_sector*>& cols, int M, bool planes, int schedule = 0);
 int krylov_upload(Krylov& K, cudaStream_t st);  // after editing hdesc (tau, out, overlaps)
 void krylov_free(Krylov& K);
-int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n, int group = -1);
+int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n, int group = -1,
+              int threads = kThreads, size_t smem = 0, int min_run = kThreads);
 
 // ----------------------------------------------------------- launchers
 // y = H x (plain); exact-hop-sum sectors use the sector's own scratch.
@@ -313,6 +314,9 @@ struct StepRunner {
     void release();
 };
 
+// KG_OK, or the status a column's kernels reported (non-finite value, device
+// wait run out) with the error message set.
+int column_rc(int status, const char* what);
 int ground_state(kg_sector* s, const kg_opts* o);
 int green_equilibrium(kg_sector* s, const int* orb, int n_orb, double dt, int n_steps, const kg_opts* o,
                       double* G_gtr, double* G_les);
@@ -526,16 +530,65 @@ __device__ __forceinline__ int4 fix_image(double2 u, int E) {
 // spare over FP64), and converts on the fly otherwise.
 constexpr int kFixSlack = 4;
 
+// Shared-memory barriers and bulk asynchronous copies (global to shared, any
+// multiple of 16 bytes between 16-byte aligned addresses).
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_init_fence() {
+    asm volatile("fence.mbarrier_init.release.cluster;\n\tfence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+// Barrier `id` (1 to 15) of the block's first `threads` threads.
+__device__ __forceinline__ void block_bar(int id, int threads) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_addr(dst)),
+                 "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_addr(bar))
+                 : "memory");
+}
+// Waits until the barrier's phase `parity` has completed; false when it has
+// not after kWaitNs or kWaitTries polls.
+constexpr int kWaitTries = 1 << 24;
+constexpr unsigned long long kWaitNs = 1000000000ull;
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
+    unsigned long long t0 = 0;
+    for (int i = 0; i < kWaitTries; ++i) {
+        unsigned done;
+        if ((i & 63) == 63) {
+            unsigned long long now;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitNs) return false;
+        }
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
 // Sum of n partials and the largest of their exponents, in a fixed order, for
 // every thread of the block (every block of a launch gets the same bits).
-// sm: 2 * (blockDim / 32) doubles.
+// sm: kThreads / 32 entries.
 __device__ __forceinline__ Partial sum_partials(const Partial* p, int n, Partial* sm) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = min((int)blockDim.x, kThreads) >> 5;
     const int used = min(nw, (n + 31) >> 5);  // warps with anything to add
     double s = 0.0;
     int e = 0;
     if (warp < used) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        for (int i = threadIdx.x; i < n; i += 32 * nw) {
             const Partial q = p[i];
             s += q.v;
             e = max(e, (int)q.e);

@@ -58,6 +58,7 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
         ColDesc& D = K.hdesc[b];
         std::memset(&D, 0, sizeof D);
         D.d = (int)s->d;
+        D.M = M;
         K.hsec[b] = s->view();
         const SecView& S = K.hsec[b];
         D.mode = S.hopmode == 0 ? ((int_hops && S.fix_pre >= 0) ? 3 : 0) : S.hopmode;
@@ -74,6 +75,7 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
     // d over the batch or over the column's group, whichever is larger
     K.group.assign(K.B, 0);
     std::vector<long long> gbytes, gd;
+    std::vector<int> slot(K.B);  // global group slot of each column
     {
         // balanced: as few groups as the budget allows, filled to the mean
         long long mbytes[4] = {0, 0, 0, 0};
@@ -97,16 +99,15 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
             }
             gbytes[cur[D.mode]] += bytes;
             gd[cur[D.mode]] += D.d;
-            D.pad = cur[D.mode];  // global group slot, used below only
+            slot[b] = cur[D.mode];
         }
     }
     np = 0;
     for (int b = 0; b < K.B; ++b) {
         ColDesc& D = K.hdesc[b];
-        const double share = std::max((double)D.d / (double)K.total_d, (double)D.d / (double)gd[D.pad]);
+        const double share = std::max((double)D.d / (double)K.total_d, (double)D.d / (double)gd[slot[b]]);
         const long long want = (long long)std::ceil(16.0 * nsm * share) + 2;
         D.nblk_max = (int)std::max(1LL, std::min(want, (long long)(D.d + kThreads - 1) / kThreads));
-        D.pad = 0;
         np += (size_t)D.nblk_max * kPart;
     }
     // on any failure the workspace is released whole (krylov_free skips null)
@@ -135,7 +136,10 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
         cudaGetLastError();
         K.Ibuf = nullptr;
     }
-    KG_TRY(need(cudaMalloc(&K.Wbuf, sizeof(double2) * 2 * nw), "work vector allocation"));
+    // U = W - a_j v_j overwrites W, except for the FP64 dots, whose thread
+    // groups each read W
+    const bool inplace = K.Ibuf != nullptr;
+    KG_TRY(need(cudaMalloc(&K.Wbuf, sizeof(double2) * (inplace ? 1 : 2) * nw), "work vector allocation"));
     if (nx) KG_TRY(need(cudaMalloc(&K.Xfbuf, sizeof(longlong2) * nx), "fixed-point image allocation"));
     KG_TRY(need(cudaMalloc(&K.partbuf, sizeof(double) * np), "partial-sum allocation"));
     KG_TRY(need(cudaMalloc(&K.pairbuf, sizeof(Partial) * 2 * (np / kPart)), "partial-sum allocation"));
@@ -160,7 +164,7 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
             ox += (size_t)D.d;
         }
         D.W = K.Wbuf + ow;
-        D.U = K.Wbuf + nw + ow;
+        D.U = inplace ? D.W : K.Wbuf + nw + ow;
         D.part = K.partbuf + op;
         D.part_a = K.pairbuf + 2 * (op / kPart);
         D.part_n = D.part_a + D.nblk_max;
@@ -205,25 +209,27 @@ void krylov_free(Krylov& K) {
     K = Krylov();
 }
 
-static int occupancy(const void* kern) {
+static int occupancy(const void* kern, int threads, size_t smem) {
     static std::mutex mu;
-    static std::map<const void*, int> occ;
+    static std::map<std::pair<const void*, size_t>, int> occ;
     std::lock_guard<std::mutex> lk(mu);
-    auto it = occ.find(kern);
+    auto it = occ.find({kern, smem});
     if (it != occ.end()) return it->second;
     int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kThreads, 0) != cudaSuccess || bps < 1) bps = 1;
-    occ[kern] = bps;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads, smem) != cudaSuccess || bps < 1) bps = 1;
+    occ[{kern, smem}] = bps;
     return bps;
 }
 
 // Work list of a kernel over the columns whose mode is `mode` (-1: all) and,
 // with group >= 0, whose H*psi group is `group`: column b gets blocks in
-// proportion to its dimension, one wave in total.
-int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n, int group) {
-    const int bps = occupancy(kern);
+// proportion to its dimension, one wave in total, with at least min_run
+// elements per block (kThreads: the kernel keeps a partial-sum row per block).
+int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n, int group, int threads, size_t smem,
+              int min_run) {
+    const int bps = occupancy(kern, threads, smem);
     const long long key = ((long long)bps << 8) + (mode + 1) + ((long long)std::lround(K.wave_scale * 64.0) << 20) +
-                          ((long long)(group + 1) << 32);
+                          ((long long)(group + 1) << 32) + ((long long)(min_run != kThreads) << 16);
     auto it = K.lists.find(key);
     if (it == K.lists.end()) {
         auto take = [&](const ColDesc& D, int b) {
@@ -238,7 +244,8 @@ int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n,
             const ColDesc& D = K.hdesc[b];
             if (!take(D, b)) continue;
             int nb = (int)std::lround(total * (double)D.d / (double)std::max(1LL, dsel));
-            nb = std::max(1, std::min(nb, std::min(D.nblk_max, (D.d + kThreads - 1) / kThreads)));
+            nb = std::max(1, std::min(nb, (D.d + min_run - 1) / min_run));
+            if (min_run == kThreads) nb = std::min(nb, D.nblk_max);
             for (int k = 0; k < nb; ++k) v.push_back(make_int4(b, k, nb, 0));
         }
         int4* d = nullptr;
@@ -292,6 +299,8 @@ __global__ void __launch_bounds__(kThreads) k_colnorm(const ColDesc* desc, const
             C->m_eff = 0;
         }
     }
+    if (blk == 0)  // totals of the exact dots of j = 0
+        for (int q = threadIdx.x; q < 4 * (D.M + 1); q += blockDim.x) D.gacc[q] = 0ull;
 }
 
 int launch_colnorm(Krylov& K, cudaStream_t st) {
@@ -421,82 +430,164 @@ __global__ void __launch_bounds__(kThreads, 2) k_reorth_dots(const ColDesc* desc
 // bound eimg[k]); u is formed in FP64 here and converted on a bound E_u of
 // its largest exponent.  With both numbers split into 26-bit halves, every
 // partial product (hi*hi, hi*lo, lo*hi, lo*lo) is an exact 64-bit integer
-// (one wide integer multiply-add).  The hi*hi and cross products are summed
-// exactly in two 64-bit accumulators (units 2^52 and 2^26 of the full
-// product); only lo*lo is rounded to the nearest 2^26, an error of 2^-79 of
-// the product of the two vectors' largest components per element.  A
-// thread's sums are converted to FP64 once per tile and reduced in a fixed
-// order.  The FP64 pipe of this GPU issues
+// (one wide integer multiply-add), summed in three 64-bit accumulators (units
+// 2^52, 2^26 and 1 of the full product).  Every further sum is an integer too:
+// over a warp in 26-bit pieces (one warp-reduce instruction each), over the
+// blocks by 64-bit atomic adds of two 46-bit limbs into gacc (in units of
+// 2^26: the rest is dropped once per warp, below 2^-79 of the product of the
+// two vectors' largest components).  Integer sums do not depend on the order, so the result is the
+// same bits on every run without a last-block reduction, and the update that
+// follows converts each total to FP64 once.  The FP64 pipe of this GPU issues
 // about 2 multiply-adds per clock per SM, the integer pipe far more, so these
 // dots are bounded by the 16 bytes of I_k per element and vector instead of
 // the 3 FP64 multiply-adds per complex product of the Re+Im form.
 //
-// Each block takes its elements in tiles of kIntTile: first every thread
-// forms kIntTile / kThreads elements of u and their images (shared memory),
-// then the G thread groups take the tile's elements for their KH vectors
-// each, the loads of an element's KH vectors issued first.
+// A block owns one run of elements and streams the NK images of it through a
+// ring of shared-memory stages filled by bulk asynchronous copies (one per
+// vector and tile; any run of 16-byte elements is a legal copy), so up to 90 KB
+// per block are in flight without holding registers.  One warp only issues the
+// copies.  The others meet once per kThreads elements, when every thread has
+// formed its element of the next u and the image of it (W and V_j of it loaded
+// one round ahead); within that round each warp walks the tiles on its own and
+// reports a tile it is done with on the stage's second barrier, which the
+// copying warp waits for before it refills the stage.  All waits are bounded;
+// after one that ran out the thread waits no more and the column's status says
+// so.
+//
+// Measured on 12 columns of 731,808 states, mean over j < 20: 529 us per launch
+// with per-thread loads, a barrier per tile and a last-block reduction; 382 us
+// (5.0 TB/s of images) in this form.  On 300 states 20 -> 10 us.  Three or more
+// vectors per warp leave too few warps to hide the multiply-adds' latency
+// (491 us), a computing warp that also refills the stages holds up the others
+// at the round's end (466 us).
 //
 // The update writes I_{j+1} on an exponent bounded before V_{j+1} exists.
 // Near a breakdown (||V_{j+1}|| far below ||W||) that bound is loose and the
 // image keeps too few of V_{j+1}'s own bits; a vector whose bound exceeds
 // its true largest exponent by more than kFixSlack bits is therefore
 // converted here from V_k on its exact exponent, the fresh image is stored
-// back (each block its own elements) and its exponent updated at the end.
-constexpr int kIntTile = 1024;
-
+// back (each block its own elements) and its exponent updated by the update.
 template <int NK>
 struct IntDots {
-    static constexpr int G = NK <= 3 ? 1 : (NK <= 6 ? 2 : (NK <= 12 ? 4 : 8));  // groups splitting k
-    static constexpr int KH = (NK + G - 1) / G;                                  // vectors per group
-    static constexpr int TG = kThreads / G;                                      // threads per group
+    // Two vectors per warp: the accumulators stay at 24 registers per thread,
+    // so that 16 to 28 warps per SM hide the latency of the multiply-adds; small
+    // NK takes several warps per vector pair.
+    static constexpr int KH = NK < 2 ? 1 : 2;           // vectors per group
+    static constexpr int G = (NK + KH - 1) / KH;        // groups splitting k
+    static constexpr int W = (8 + G - 1) / G;           // warps per group
+    static constexpr int TG = 32 * W;                   // threads per group
+    static constexpr int compute = TG * G;              // 256 to 448 threads per block
+    static constexpr int threads = compute + 32;        // and the warp that issues the copies
+    static constexpr int T = NK <= 6 ? 256 : (NK <= 12 ? 128 : 64);  // elements per tile
+    static constexpr int kStage = NK * T * 16;
+    static constexpr int kImage = 2 * kThreads * 24;  // two rounds of u's image
+    static constexpr int fit = (104 * 1024 - kImage) / kStage;
+    static constexpr int S = fit > 8 ? 8 : fit;  // stages; two blocks per SM
+    static constexpr size_t smem = (size_t)S * kStage + kImage;
+    static_assert(S >= 3, "at least three stages");
 };
 
+constexpr int kDotFlush = 256;   // elements a thread may add to its 64-bit sums
+constexpr int kDotMinRun = 64;   // fewest elements worth a block
+
 // Re and Im of conj(v) u for v and u given as split 52-bit images (v:
-// {x_hi, x_lo, y_hi, y_lo}; u: Re hi/lo, Im hi/lo and -Re hi/lo): the
-// hi*hi part in units of 2^52 (re2, im2) and the rest in units of 2^26
-// (re1, im1) of the full product.
-__device__ __forceinline__ void cdot_fix(const int4 v, const int* uw, long long& re2, long long& re1,
-                                         long long& im2, long long& im1) {
-    const int p1 = uw[0], p0 = uw[1], q1 = uw[2], q0 = uw[3], n1 = uw[4], n0 = uw[5];
+// {x_hi, x_lo, y_hi, y_lo}; u likewise, m: hi and lo of -Re u), added to sums
+// in units of 2^52 (s[0]), 2^26 (s[1]) and 1 (s[2]) of the full product.
+__device__ __forceinline__ void cdot_fix(const int4 v, const int4 u, const int2 m, long long (&re)[3],
+                                         long long (&im)[3]) {
+    const int p1 = u.x, p0 = u.y, q1 = u.z, q0 = u.w, n1 = m.x, n0 = m.y;
     // Re = vx ux + vy uy
-    re2 += (long long)v.x * p1 + (long long)v.z * q1;
-    re1 += (long long)v.x * p0 + (long long)v.y * p1 + (long long)v.z * q0 + (long long)v.w * q1 +
-           (((long long)v.y * p0 + (long long)v.w * q0 + (1ll << 25)) >> 26);
+    re[0] += (long long)v.x * p1 + (long long)v.z * q1;
+    re[1] += (long long)v.x * p0 + (long long)v.y * p1 + (long long)v.z * q0 + (long long)v.w * q1;
+    re[2] += (long long)v.y * p0 + (long long)v.w * q0;
     // Im = vx uy - vy ux
-    im2 += (long long)v.x * q1 + (long long)v.z * n1;
-    im1 += (long long)v.x * q0 + (long long)v.y * q1 + (long long)v.z * n0 + (long long)v.w * n1 +
-           (((long long)v.y * q0 + (long long)v.w * n0 + (1ll << 25)) >> 26);
+    im[0] += (long long)v.x * q1 + (long long)v.z * n1;
+    im[1] += (long long)v.x * q0 + (long long)v.y * q1 + (long long)v.z * n0 + (long long)v.w * n1;
+    im[2] += (long long)v.y * q0 + (long long)v.w * n0;
+}
+
+// The warp's total of s[0] 2^26 + s[1] + s[2] 2^-26 (|s[0]| < 2^62) as two
+// limbs, total = l1 2^46 + l0.
+__device__ __forceinline__ void warp_limbs(const long long (&s)[3], unsigned long long& l0, unsigned long long& l1) {
+    constexpr long long m26 = (1ll << 26) - 1;
+    const long long lo = s[1] + (s[2] >> 26), hi = s[0] + (lo >> 26);
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)(lo & m26));
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(hi & m26));
+    const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)((hi >> 26) & m26));
+    const int s3 = __reduce_add_sync(0xffffffffu, (int)(hi >> 52));
+    const unsigned long long a = (unsigned long long)s0 + ((unsigned long long)s1 << 26);   // < 2^58
+    const long long b = (long long)s2 + ((long long)s3 << 26);                               // units of 2^52
+    l0 = a & ((1ull << 46) - 1ull);
+    l1 = (unsigned long long)((b << 6) + (long long)(a >> 46));
 }
 
 template <int NK>
-__global__ void __launch_bounds__(kThreads, 3) k_reorth_dots_int(const ColDesc* desc, const int4* items,
-                                                                 ColScalars* cs, int j, int k0, int nk,
-                                                                 unsigned* cnt) {
-    constexpr int G = IntDots<NK>::G, KH = IntDots<NK>::KH, TG = IntDots<NK>::TG;
-    constexpr int R = kIntTile / kThreads;         // elements of u per thread and tile
-    __shared__ int up[kIntTile][6];                // image of u: Re hi/lo, Im hi/lo, -Re hi/lo
-    __shared__ double sm[(kThreads / 32) * 2 * KH];
-    __shared__ double bs[2 * NK], red[2 * NK];
-    __shared__ int eu_s;
-    __shared__ int fresh_s[NK], ek_s[NK];
+__global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(const ColDesc* desc, const int4* items,
+                                                                 ColScalars* cs, int j, int k0) {
+    using P = IntDots<NK>;
+    constexpr int KH = P::KH, TG = P::TG, T = P::T, S = P::S;
+    extern __shared__ __align__(128) unsigned char dyn[];
+    __shared__ __align__(8) unsigned long long full[S], empty[S];
     __shared__ Partial pair[kThreads / 32];
+    __shared__ int eu_s, any_s, fresh_s[NK], ek_s[NK];
+    int4* const ua = reinterpret_cast<int4*>(dyn + S * P::kStage);  // [2][kThreads] image of u
+    int2* const ub = reinterpret_cast<int2*>(dyn + S * P::kStage + 2 * kThreads * 16);
     KG_ITEM();
     if (j >= C->m_eff) return;
-    int ew;
-    const double araw = resolve_alpha(D, C, blk == 0 && threadIdx.x == 0, pair, ew);
     const int d = D.d;
-    const int grp = threadIdx.x / TG, t = threadIdx.x % TG;
-    const int kb = grp * KH, kn = min(KH, NK - kb);
-    int4* Ib = D.I + (size_t)(k0 + kb) * d;
-    const double2* Vk = D.V + (size_t)(k0 + kb) * d;
-    const double2* w = D.W;
-    const double2* vj = D.V + (size_t)j * d;
+    // this block's elements [e0, e0 + len), in tiles of T
+    const int run = (int)(((long long)d + nblk - 1) / nblk);
+    const size_t e0 = (size_t)min((long long)d, (long long)blk * run);
+    const int len = (int)min((long long)run, (long long)d - (long long)e0);
+    const int nt = (len + T - 1) / T, nr = (len + kThreads - 1) / kThreads;
+    const int4* Ib = D.I + (size_t)k0 * d + e0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+            mbar_init(full + q, 1);
+            mbar_init(empty + q, P::compute / 32);
+        }
+        mbar_init_fence();
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const bool copies = threadIdx.x >= P::compute;
+    auto issue = [&](int t) {  // by the copying warp: tile t into its stage
+        const int q = t % S, n = min(T, len - t * T);
+        if (lane == 0) mbar_expect(full + q, (unsigned)(NK * n * 16));
+        __syncwarp();
+        if (lane < NK)
+            bulk_load(dyn + q * P::kStage + lane * T * 16, Ib + (size_t)lane * d + (size_t)t * T, (unsigned)(n * 16),
+                      full + q);
+    };
+    if (copies)
+        for (int t = 0; t < min(S, nt); ++t) issue(t);
+    double2 wn = make_double2(0.0, 0.0), vn = wn;  // W and V_j of this thread's element of the next round
+    const double2* wp = D.W + e0;
+    const double2* vp = D.V + (size_t)j * d + e0;
+    auto load_u = [&](int r) {
+        const int e = r * kThreads + (int)threadIdx.x;
+        if (threadIdx.x < kThreads && e < len) {
+            wn = wp[e];
+            vn = vp[e];
+        }
+    };
+    if (nr > 0) load_u(0);
+    const bool writer = blk == 0 && threadIdx.x == 0;
+    int ew;
+    const double araw = resolve_alpha(D, C, writer, pair, ew);
     const double aj = araw * C->scale[j];
-    // the last chunk leaves u = W - a_j v_j in U
+    // the last chunk leaves u = W - a_j v_j in U (which may be W itself)
     const bool keep = k0 + NK == j + 1;
     if (threadIdx.x < NK) {
         ek_s[threadIdx.x] = C->emax[k0 + threadIdx.x];
         fresh_s[threadIdx.x] = C->eimg[k0 + threadIdx.x] - C->emax[k0 + threadIdx.x] > kFixSlack;
+    }
+    if (threadIdx.x < 32) {
+        __syncwarp();
+        const bool f = threadIdx.x < NK && fresh_s[threadIdx.x < NK ? threadIdx.x : 0];
+        const unsigned any = __ballot_sync(0xffffffffu, f);
+        if (threadIdx.x == 0) any_s = any != 0u;
     }
     if (threadIdx.x == 0) {
         // |u_i| <= |W_i| + |a_j| |V_j[i]| < (1 + |a_j| 2^(E_j - E_w)) 2^(E_w - 1022), with a margin
@@ -504,87 +595,93 @@ __global__ void __launch_bounds__(kThreads, 3) k_reorth_dots_int(const ColDesc* 
         int ex;
         const double fr = frexp(r, &ex);
         eu_s = ew + (fr == 0.5 ? ex - 1 : ex);
+        if (writer) C->eu = eu_s;
     }
     __syncthreads();
     const int Eu = eu_s;
-    double acc[2 * KH];
-#pragma unroll
-    for (int q = 0; q < 2 * KH; ++q) acc[q] = 0.0;
-    auto load = [&](int k, int i) -> int4 {
-        if (fresh_s[kb + k]) {
-            const int4 v = fix_image(Vk[(size_t)k * d + i], ek_s[kb + k]);
-            Ib[(size_t)k * d + i] = v;
-            return v;
+    const bool any_fresh = any_s != 0;
+    const int grp = threadIdx.x / TG, tl = threadIdx.x % TG;
+    const int kb = grp * KH, kn = min(KH, NK - kb);
+    bool ok = true;
+    if (copies) {
+        for (int t = S; t < nt && ok; ++t) {  // the tile that held the stage before is done with
+            ok = mbar_wait(empty + t % S, (unsigned)((t / S - 1) & 1));
+            if (ok) issue(t);
         }
-        return Ib[(size_t)k * d + i];
+        for (int t = max(0, nt - S); t < nt && ok; ++t) ok = mbar_wait(full + t % S, (unsigned)((t / S) & 1));
+        if (!ok) C->status = KG_ETIMEOUT;
+        return;
+    }
+    double2* const up = D.U + e0;
+    auto form_u = [&](int r) {
+        const int e = r * kThreads + (int)threadIdx.x;
+        if (threadIdx.x >= kThreads || e >= len) return;
+        const double2 u = make_double2(fma(-aj, vn.x, wn.x), fma(-aj, vn.y, wn.y));
+        if (keep) up[e] = u;
+        const long long px = fix52(u.x, Eu), py = fix52(u.y, Eu);
+        const int at = (r & 1) * kThreads + (int)threadIdx.x;
+        ua[at] = make_int4(fix_hi(px), fix_lo(px), fix_hi(py), fix_lo(py));
+        ub[at] = make_int2(fix_hi(-px), fix_lo(-px));
     };
-    for (int base = blk * kIntTile; base < d; base += nblk * kIntTile) {
+    long long re[KH][3], im[KH][3];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int e = threadIdx.x + r * kThreads, i = base + e;
-            if (i < d) {
-                double2 u = w[i];
-                const double2 p = vj[i];
-                u.x = fma(-aj, p.x, u.x);
-                u.y = fma(-aj, p.y, u.y);
-                if (keep) D.U[i] = u;
-                const long long px = fix52(u.x, Eu), py = fix52(u.y, Eu);
-                up[e][0] = fix_hi(px);
-                up[e][1] = fix_lo(px);
-                up[e][2] = fix_hi(py);
-                up[e][3] = fix_lo(py);
-                up[e][4] = fix_hi(-px);
-                up[e][5] = fix_lo(-px);
-            }
-        }
-        __syncthreads();
-        const int end = min(kIntTile, d - base);
-        long long re2[KH], re1[KH], im2[KH], im1[KH];
+    for (int k = 0; k < KH; ++k)
 #pragma unroll
-        for (int k = 0; k < KH; ++k) re2[k] = re1[k] = im2[k] = im1[k] = 0;
-        // a thread takes kIntTile / TG <= 32 elements of the tile, each adding
-        // at most 2^54.1 to an accumulator: the sums stay below 2^60
-        for (int e = t; e < end; e += TG) {
-            int4 va[KH];
-#pragma unroll
-            for (int k = 0; k < KH; ++k)
-                if (k < kn) va[k] = load(k, base + e);
-#pragma unroll
-            for (int k = 0; k < KH; ++k)
-                if (k < kn) cdot_fix(va[k], up[e], re2[k], re1[k], im2[k], im1[k]);
-        }
+        for (int q = 0; q < 3; ++q) re[k][q] = im[k][q] = 0;
+    int held = 0;  // elements in the sums
+    unsigned long long* const acc = D.gacc + (size_t)(j & 1) * 4 * (D.M + 1) + 4 * (size_t)(k0 + kb);
+    auto flush = [&]() {
+        unsigned long long l0 = 0, l1 = 0;
 #pragma unroll
         for (int k = 0; k < KH; ++k) {
-            acc[2 * k] += fma((double)re1[k], 0x1p-26, (double)re2[k]);
-            acc[2 * k + 1] += fma((double)im1[k], 0x1p-26, (double)im2[k]);
-        }
-        __syncthreads();
-    }
-    // block sums: warps reduce, then each group's warps in warp order
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+            unsigned long long a0, a1;
+            warp_limbs(re[k], a0, a1);
+            if (lane == 2 * k) l0 = a0, l1 = a1;
+            warp_limbs(im[k], a0, a1);
+            if (lane == 2 * k + 1) l0 = a0, l1 = a1;
 #pragma unroll
-    for (int q = 0; q < 2 * KH; ++q) {
-        const double v = warp_sum(acc[q]);
-        if (lane == 0) sm[warp * 2 * KH + q] = v;
-    }
-    __syncthreads();
-    constexpr int WG = TG / 32;  // warps per group
-    for (int q = threadIdx.x; q < 2 * NK; q += blockDim.x) {
-        const int g = q / (2 * KH), l = q - g * 2 * KH;
-        double sum = 0.0;
-        for (int w2 = 0; w2 < WG; ++w2) sum += sm[(g * WG + w2) * 2 * KH + l];
-        bs[q] = sum;
-    }
-    __syncthreads();
-    if (grid_finish(bs, 2 * NK, D.part, cnt + b, blk, nblk, red)) {
-        for (int k = threadIdx.x; k < NK; k += blockDim.x) {
-            // units: 2^52 of 2^(E_k - 1074) 2^(E_u - 1074), E_k the exponent of V_k's image
-            const int Ei = fresh_s[k] ? C->emax[k0 + k] : C->eimg[k0 + k];
-            const double f = C->scale[k0 + k] * ldexp(1.0, Ei + Eu - 2096);
-            C->h[k0 + k] = make_double2(f * red[2 * k], f * red[2 * k + 1]);
-            C->eimg[k0 + k] = Ei;
+            for (int q = 0; q < 3; ++q) re[k][q] = im[k][q] = 0;
         }
+        if (lane < 2 * kn) {
+            atomicAdd(acc + 2 * lane, l0);
+            atomicAdd(acc + 2 * lane + 1, l1);
+        }
+        held = 0;
+    };
+    if (nr > 0) form_u(0);
+    block_bar(1, P::compute);
+    int t = 0;
+    for (int r = 0; r < nr; ++r) {
+        if (r + 1 < nr) load_u(r + 1);
+        const int tend = min(nt, (r + 1) * (kThreads / T));
+        for (; t < tend; ++t) {
+            ok = ok && mbar_wait(full + t % S, (unsigned)((t / S) & 1));
+            int4* img = reinterpret_cast<int4*>(dyn + (t % S) * P::kStage) + kb * T;
+            const int n = min(T, len - t * T), base = (r & 1) * kThreads + (t * T) % kThreads;
+            if (any_fresh)  // re-made images replace what was copied (each thread its own elements)
+                for (int k = 0; k < kn; ++k)
+                    for (int e = tl; fresh_s[kb + k] && e < n; e += TG) {
+                        const size_t at = (size_t)(k0 + kb + k) * d + e0 + (size_t)t * T + e;
+                        img[k * T + e] = D.I[at] = fix_image(D.V[at], ek_s[kb + k]);
+                    }
+#pragma unroll 2
+            for (int e = tl; e < n; e += TG) {
+                const int4 u = ua[base + e];
+                const int2 m = ub[base + e];
+#pragma unroll
+                for (int k = 0; k < KH; ++k)
+                    if (k < kn) cdot_fix(img[k * T + e], u, m, re[k], im[k]);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + t % S);
+        }
+        held += (kThreads + TG - 1) / TG;
+        if (held > kDotFlush - (kThreads + TG - 1) / TG) flush();
+        if (r + 1 < nr) form_u(r + 1);
+        block_bar(1, P::compute);
     }
+    flush();
+    if (!ok) C->status = KG_ETIMEOUT;
 }
 
 // The accumulators of k_reorth_dots are compile-time sized and a kernel
@@ -603,17 +700,30 @@ static DotsKernel dots_kernel(int nk) {
     return exact[nk - 1];
 }
 
-using IntDotsKernel = void (*)(const ColDesc*, const int4*, ColScalars*, int, int, int, unsigned*);
+struct IntDotsKernel {
+    void (*kern)(const ColDesc*, const int4*, ColScalars*, int, int);
+    int threads;
+    size_t smem;
+};
 
 template <int... N>
-static constexpr std::array<IntDotsKernel, sizeof...(N)> int_dots_table(std::integer_sequence<int, N...>) {
-    return {{&k_reorth_dots_int<N + 1>...}};
+static std::array<IntDotsKernel, sizeof...(N)> int_dots_table(std::integer_sequence<int, N...>) {
+    const std::array<IntDotsKernel, sizeof...(N)> t = {{{&k_reorth_dots_int<N + 1>, IntDots<N + 1>::threads, IntDots<N + 1>::smem}...}};
+    for (auto& k : t)
+        cudaFuncSetAttribute((const void*)k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    return t;
 }
 
+// Per device: the shared-memory attribute belongs to the device's context.
 static IntDotsKernel int_dots_kernel(int nk) {
-    static const std::array<IntDotsKernel, kChunk> exact =
-        int_dots_table(std::make_integer_sequence<int, kChunk>{});
-    return exact[nk - 1];
+    static std::mutex mu;
+    static std::map<int, std::array<IntDotsKernel, kChunk>> tables;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = tables.find(dev);
+    if (it == tables.end()) it = tables.emplace(dev, int_dots_table(std::make_integer_sequence<int, kChunk>{})).first;
+    return it->second[nk - 1];
 }
 
 // The exact integer dots serve first passes when every column has its images.
@@ -630,8 +740,8 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
         const IntDotsKernel ik = int_dots_kernel(nk);
         const int4* items;
         int n;
-        KG_TRY(work_list(K, (const void*)ik, -1, &items, &n));
-        ik<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, k0, nk, K.cnt);
+        KG_TRY(work_list(K, (const void*)ik.kern, -1, &items, &n, -1, ik.threads, ik.smem, kDotMinRun));
+        ik.kern<<<n, ik.threads, ik.smem, st>>>(K.desc, items, K.cs, j, k0);
         KG_LAUNCHED();
         return KG_OK;
     }
@@ -659,18 +769,34 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
 // than the FP64 pipe on this GPU.  Larger coefficients use FP64.
 constexpr double kSmallCoef = 1e-10;
 
+// h_k = s_k <V_k, u> from the exact integer totals of the dots (units 2^26 of
+// 2^(E_k - 1074) 2^(E_u - 1074), E_k the exponent of V_k's image; `keep`: also
+// store E_k, which the dots changed if they re-made the image).
+__device__ __forceinline__ double2 exact_dot(const ColDesc& D, ColScalars* C, int j, int k, bool keep) {
+    const ulonglong2* t = reinterpret_cast<const ulonglong2*>(D.gacc + (size_t)(j & 1) * 4 * (D.M + 1) + 4 * (size_t)k);
+    const int em = C->emax[k], ei = C->eimg[k], Ek = ei - em > kFixSlack ? em : ei;
+    const double f = C->scale[k] * ldexp(1.0, Ek + C->eu - 2122);
+    auto val = [](ulonglong2 l) {
+        const long long hi = (long long)l.y + (long long)(l.x >> 46);
+        return fma((double)hi, 0x1p46, (double)(l.x & ((1ull << 46) - 1ull)));
+    };
+    if (keep) C->eimg[k] = Ek;
+    return make_double2(f * val(t[0]), f * val(t[1]));
+}
+
 // Its first warp sorts the terms, one vector per lane: a serial pass by one
 // thread costs two dependent L2 reads and a few FP64 operations per vector in
 // every block.  With the sums reduced by the reader (resolve_norm) instead of
 // by the last block to arrive, a Lanczos iteration on a 300-state column at
 // M = 40 went from 53 to 38 us, on one 853,776-state column from 190 to 174 us.
 __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const int4* items, ColScalars* cs, int j,
-                                                     int level, int second) {
+                                                     int level, int second, int exact) {
     // block-uniform term lists: FP32 terms (small coefficients), FP64 terms
     __shared__ double2 coef64[kMaxMgs + 1];
     __shared__ float2 coef32[kMaxMgs + 1];
     __shared__ int idx32[kMaxMgs + 1], idx64[kMaxMgs + 1];
     __shared__ int n32, n64, efix_s;
+    __shared__ double hre_s;
     __shared__ double sm[kThreads / 32];
     __shared__ int smi[kThreads / 32];
     __shared__ Partial pair[kThreads / 32];
@@ -703,7 +829,8 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
             double2 h = make_double2(0.0, 0.0), c = h;
             if (k < nk) {
                 const double s = C->scale[k];
-                h = C->h[k];
+                h = exact ? exact_dot(D, C, j, k, blk == 0) : C->h[k];
+                if (k == j) hre_s = h.x;
                 c = make_double2(s * h.x, s * h.y);
                 r += (fabs(c.x) + fabs(c.y)) * ldexp(1.0, C->emax[k] - ew);
             }
@@ -849,8 +976,11 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     if (writer) {
         C->n_norm = nblk;
         C->abase = second ? C->alpha[j] : araw;
-        C->hre = nk ? C->h[j].x : 0.0;
+        C->hre = nk ? hre_s : 0.0;
     }
+    // the other parity's totals are free: cleared for the dots of j + 1
+    if (exact && blk == 0)
+        for (int q = threadIdx.x; q < 4 * (D.M + 1); q += blockDim.x) D.gacc[((j + 1) & 1) * 4 * (D.M + 1) + q] = 0ull;
 }
 
 // resolve_norm by itself, one block per column.
@@ -872,7 +1002,8 @@ int launch_update(Krylov& K, int j, int level, bool second, cudaStream_t st) {
     const int4* items;
     int n;
     KG_TRY(work_list(K, (const void*)k_update, -1, &items, &n));
-    k_update<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, level, second ? 1 : 0);
+    const int exact = level >= 1 && use_int_dots(K, second);
+    k_update<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, level, second ? 1 : 0, exact);
     KG_LAUNCHED();
     return KG_OK;
 }
@@ -1438,7 +1569,10 @@ int prepare_step(Krylov& K, int reorth) {
         // every vector count of one step (and of the ground-state restarts)
         for (int nk = 1; nk <= std::min(kChunk, K.M + 1); ++nk) {
             KG_TRY(work_list(K, (const void*)dots_kernel(nk), -1, &items, &n));
-            if (use_int_dots(K, false)) KG_TRY(work_list(K, (const void*)int_dots_kernel(nk), -1, &items, &n));
+            if (use_int_dots(K, false)) {
+                const IntDotsKernel ik = int_dots_kernel(nk);
+                KG_TRY(work_list(K, (const void*)ik.kern, -1, &items, &n, -1, ik.threads, ik.smem, kDotMinRun));
+            }
         }
     }
     const void* comb[4] = {(const void*)k_combine<0>, (const void*)k_combine<4>, (const void*)k_combine<12>,
@@ -1471,6 +1605,13 @@ int enqueue_step(Krylov& K, int reorth, cudaStream_t st) {
     KG_TRY(launch_tridiag(K, 0, st));
     KG_TRY(launch_combine(K, st));
     return KG_OK;
+}
+
+int column_rc(int status, const char* what) {
+    if (status == KG_ENUMERIC) set_error("non-finite value during %s", what);
+    else if (status == KG_ETIMEOUT) set_error("a bounded device wait ran out during %s", what);
+    else return KG_OK;
+    return status;
 }
 
 // ------------------------------------------------------ ground state
@@ -1513,7 +1654,8 @@ int ground_state(kg_sector* s, const kg_opts* o) {
             rc = cuda_fail(cudaGetLastError(), "ground-state readback", __FILE__, __LINE__);
             break;
         }
-        if (h.status == KG_ENUMERIC || !(h.ovnorm > 0.0) || !std::isfinite(h.ovnorm)) {
+        if ((rc = column_rc(h.status, "the ground-state Lanczos recursion")) != KG_OK) break;
+        if (!(h.ovnorm > 0.0) || !std::isfinite(h.ovnorm)) {
             set_error("non-finite value in the ground-state Lanczos recursion");
             rc = KG_ENUMERIC;
             break;

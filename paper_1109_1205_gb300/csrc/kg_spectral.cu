@@ -73,10 +73,7 @@ static int lanczos_columns(kg_sector* s, const int* orb, int n_orb, int n, const
     krylov_free(K);
     if (rc != KG_OK) return rc;
     for (auto& c : h)
-        if (c.status == KG_ENUMERIC) {
-            set_error("non-finite value in the Lanczos run");
-            return KG_ENUMERIC;
-        }
+        KG_TRY(column_rc(c.status, "the Lanczos run"));
     return KG_OK;
 }
 
