@@ -74,7 +74,8 @@ typedef struct kg_opts {
                            may plan for; 0 = the free memory at creation (0) */
     int schedule;       /* bit 0: H*psi hop sums in FP64 always, instead of
                            exact 64-bit integer sums when all hops share one
-                           amplitude; bit 1: each propagation step's
+                           amplitude (or, in steps of small sectors, of any
+                           hops as 56-bit fixed-point products); bit 1: each propagation step's
                            exponential e^{-iT tau} e_1 through the eigen-
                            decomposition of T (Section 3, Eq. (udelta)),
                            instead of the scaled Taylor series of the same

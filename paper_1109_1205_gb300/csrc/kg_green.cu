@@ -184,7 +184,7 @@ static int eq_run(std::vector<EqGroup>& G, const std::vector<kg_sector*>& inst, 
     if (n_steps == 0) return KG_OK;
     StepRunner R;
     const bool graphs = o->use_graphs != 0;
-    if (tune && n_steps > 4 && graphs && !profiling()) {
+    if (tune && n_steps > 4 && graphs && !profiling() && !small_steps(K, o->reorth)) {
         // autotuner: work-list size relative to one wave, timed on two steps
         const double cands[3] = {0.5, 1.0, 2.0};
         double best_t = 1e300, best = 1.0;

@@ -135,36 +135,6 @@ __device__ __forceinline__ void hop_sum_pre(const SecView& S, const longlong2* _
     iy += py - ny;
 }
 
-// v * 2^(E - 1075 - P) rounded to nearest (ties to even), assembled on the
-// integer pipe: the FP64 pipe of this GPU is the scarce one.  |v| < 2^62.
-// Falls back to FP64 arithmetic if the result would be subnormal.
-__device__ __forceinline__ double fix_to_double(long long v, int E, int P) {
-    if (v == 0) return 0.0;
-    const unsigned long long sgn = (unsigned long long)v & 0x8000000000000000ull;
-    unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
-    const int n = 63 - __clzll((long long)a);  // position of the leading bit
-    int be = n + E - 52 - P;                    // biased exponent of the result
-    unsigned long long m;
-    if (n > 52) {
-        const int s = n - 52;
-        m = a >> s;
-        const unsigned long long rem = a & ((1ull << s) - 1ull), half = 1ull << (s - 1);
-        if (rem > half || (rem == half && (m & 1ull))) ++m;
-        if (m >> 53) {
-            m >>= 1;
-            ++be;
-        }
-    } else {
-        m = a << (52 - n);
-    }
-    if (be < 1) {
-        const long long ex = (long long)E - 52 - P;
-        return ex > 0 ? __ll2double_rn(v) * __longlong_as_double(ex << 52) : 0.0;
-    }
-    return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (m & 0xfffffffffffffull)));
-}
-
-
 __device__ __forceinline__ void stage_amplitudes(const SecView& S, double2* amp) {
     for (int k = threadIdx.x; k < S.L * S.L; k += blockDim.x) amp[k] = S.hamp[k];
     __syncthreads();

@@ -166,6 +166,7 @@ struct ColDesc {
     int4* I;                // [M+1][d] V_k in 52-bit fixed point on eimg[k], split
                             // into 26-bit halves {x_hi, x_lo, y_hi, y_lo} (or null)
     longlong2* Xf;          // [d] fixed-point image of the next H*psi input (or null)
+    int4* Xs;               // [d] likewise, in 28-bit halves (small columns, else null)
     double2* W;             // [d] H v workspace
     double2* U;             // [d] W - a_j v_j, left by the Gram-Schmidt dots
     double* part;           // [nblk_max][kPart] partial sums of this column
@@ -181,6 +182,7 @@ struct ColDesc {
     int mode;               // hop sums: 0 FP64 uniform, 1 real, 2 complex, 3 exact integer
     int Du, Dd, fix_pre;    // row length, row count, fixed-point pre-shift of the sector
     int M;                  // Krylov dimension of the workspace
+    int small;              // blocks of the cluster that takes whole steps of this column (0: streaming)
 };
 
 // B columns of (possibly) different sectors.  Every streaming kernel runs over
@@ -204,6 +206,18 @@ struct Krylov {
     float2* V32buf = nullptr;
     int4* Ibuf = nullptr;           // fixed-point images of the exact Gram-Schmidt dots
     longlong2* Xfbuf = nullptr;     // fixed-point H*psi inputs of exact-integer columns
+    int4* Xsbuf = nullptr;          // the same of small columns
+    // small columns (kg_small.cu), one launch per cluster size and step
+    struct SmallGroup {
+        int cluster = 1, ept = 1, n = 0;
+        size_t smem = 0;
+        int* cols = nullptr;        // [n] on the device
+        cudaStream_t side = nullptr;  // beside the other groups
+        cudaEvent_t done = nullptr;
+    };
+    std::vector<SmallGroup> small;
+    cudaEvent_t fork = nullptr;
+    bool fused = false;             // the last space came from kg_small.cu (all columns are small)
     double2* Wbuf = nullptr;
     double* partbuf = nullptr;
     Partial* pairbuf = nullptr;
@@ -224,6 +238,15 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
                  bool planes = true);
 // Device bytes krylov_alloc takes for these columns (an upper estimate).
 size_t krylov_bytes(const std::vector<const kg_sector*>& cols, int M, bool planes, int schedule = 0);
+// Batches of small columns: their cluster sizes (Krylov dimension M; all 0 for
+// the streaming kernels), the groups of equal size, and one launch per group
+// of their whole step (finish) or Lanczos space.
+void small_plan(const std::vector<const kg_sector*>& cols, int M, int schedule, std::vector<int>& cluster);
+int small_alloc(Krylov& K, const std::vector<const kg_sector*>& cols);
+void small_free(Krylov& K);
+int launch_small(Krylov& K, bool finish, cudaStream_t st);
+// Whether spaces of reorthogonalisation level `reorth` use it.
+inline bool small_steps(const Krylov& K, int reorth) { return reorth == 1 && !K.small.empty(); }
 int krylov_upload(Krylov& K, cudaStream_t st);  // after editing hdesc (tau, out, overlaps)
 void krylov_free(Krylov& K);
 int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n, int group = -1,
@@ -499,6 +522,35 @@ __device__ __forceinline__ long long fix_term(double x, int E, int P, uint32_t n
     return ((uint32_t)(b >> 63) ^ neg) ? -v : v;
 }
 
+// v * 2^(E - 1075 - P) rounded to nearest (ties to even), assembled on the
+// integer pipe: the FP64 pipe of this GPU is the scarce one.  |v| < 2^62.
+// Falls back to FP64 arithmetic if the result would be subnormal.
+__device__ __forceinline__ double fix_to_double(long long v, int E, int P) {
+    if (v == 0) return 0.0;
+    const unsigned long long sgn = (unsigned long long)v & 0x8000000000000000ull;
+    unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int n = 63 - __clzll((long long)a);  // position of the leading bit
+    int be = n + E - 52 - P;                    // biased exponent of the result
+    unsigned long long m;
+    if (n > 52) {
+        const int s = n - 52;
+        m = a >> s;
+        const unsigned long long rem = a & ((1ull << s) - 1ull), half = 1ull << (s - 1);
+        if (rem > half || (rem == half && (m & 1ull))) ++m;
+        if (m >> 53) {
+            m >>= 1;
+            ++be;
+        }
+    } else {
+        m = a << (52 - n);
+    }
+    if (be < 1) {
+        const long long ex = (long long)E - 52 - P;
+        return ex > 0 ? __ll2double_rn(v) * __longlong_as_double(ex << 52) : 0.0;
+    }
+    return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (m & 0xfffffffffffffull)));
+}
+
 // round(x * 2^(1074 - E)) for E at least the exponent field of x, so that
 // |x| < 2^(E - 1022) and |result| < 2^52: a 52-bit fixed-point number whose
 // unit is 2^-52 of the bound.  Zero and subnormal x give 0.  Integer pipe
@@ -578,6 +630,127 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
     }
     return false;
 }
+
+// A Gram-Schmidt term whose coefficient (on the unit vector) is below this is
+// subtracted in FP32 (kg_krylov.cu, the update).
+constexpr double kSmallCoef = 1e-10;
+
+// ------------------------------------ step exponential by a Taylor series
+// e^{-i T tau} e_1 for the tridiagonal T, the vector of Eq. (udelta), without
+// the eigen-decomposition: the series in (-i T h) with h = tau / n_sub and
+// n_sub chosen so that |T h| <= 1 (Gershgorin bound), 22 terms per sub-step
+// (remainder below 1e-22 of the sum).  One warp; lane l holds components l and
+// l + 32 (R = 2), so every FP64 instruction serves the whole vector -- the
+// eigen-decomposition's bulge chase is serial.  An FP64 warp instruction holds
+// its SM quarter's pipe for 64 cycles, so what counts is their number: the
+// factors h / n come from products, and the first sub-step, from the real e_1,
+// takes five per component and term instead of ten.
+constexpr int kTaylorTerms = 22;
+static __constant__ double c_taylor[kTaylorTerms] = {1.0 / 1,  1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,
+                                                     1.0 / 7,  1.0 / 8,  1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12,
+                                                     1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18,
+                                                     1.0 / 19, 1.0 / 20, 1.0 / 21, 1.0 / 22};
+
+template <int R>
+struct Tridiag {
+    double a[R], bl[R], br[R], g;  // diagonal, couplings to k - 1 and k + 1, row-sum bound
+    __device__ __forceinline__ void load(const double* alpha, const double* beta, int m, int lane) {
+        g = 0.0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int k = lane + 32 * r;
+            a[r] = k < m ? alpha[k] : 0.0;
+            bl[r] = (k < m && k >= 1) ? beta[k] : 0.0;
+            br[r] = (k + 1 < m) ? beta[k + 1] : 0.0;
+            g = fmax(g, fabs(a[r]) + fabs(bl[r]) + fabs(br[r]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
+    }
+    __device__ __forceinline__ void apply(const double2 (&x)[R], double2 (&y)[R], int lane) const {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            // x_{k-1} and x_{k+1} for k = lane + 32 r
+            double2 xm, xp;
+            xm.x = __shfl_up_sync(0xffffffffu, x[r].x, 1);
+            xm.y = __shfl_up_sync(0xffffffffu, x[r].y, 1);
+            xp.x = __shfl_down_sync(0xffffffffu, x[r].x, 1);
+            xp.y = __shfl_down_sync(0xffffffffu, x[r].y, 1);
+            if (R > 1) {
+                const double2 lo = r > 0 ? x[r > 0 ? r - 1 : 0] : make_double2(0.0, 0.0);
+                const double2 hi = r + 1 < R ? x[r + 1 < R ? r + 1 : r] : make_double2(0.0, 0.0);
+                const double lox = __shfl_sync(0xffffffffu, lo.x, 31), loy = __shfl_sync(0xffffffffu, lo.y, 31);
+                const double hix = __shfl_sync(0xffffffffu, hi.x, 0), hiy = __shfl_sync(0xffffffffu, hi.y, 0);
+                if (lane == 0) xm = make_double2(lox, loy);
+                if (lane == 31) xp = make_double2(hix, hiy);
+            }
+            y[r].x = fma(a[r], x[r].x, fma(bl[r], xm.x, br[r] * xp.x));
+            y[r].y = fma(a[r], x[r].y, fma(bl[r], xm.y, br[r] * xp.y));
+        }
+    }
+    __device__ __forceinline__ void apply(const double (&x)[R], double (&y)[R], int lane) const {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            double xm = __shfl_up_sync(0xffffffffu, x[r], 1), xp = __shfl_down_sync(0xffffffffu, x[r], 1);
+            if (R > 1) {
+                const double lo = __shfl_sync(0xffffffffu, r > 0 ? x[r > 0 ? r - 1 : 0] : 0.0, 31);
+                const double hi = __shfl_sync(0xffffffffu, r + 1 < R ? x[r + 1 < R ? r + 1 : r] : 0.0, 0);
+                if (lane == 0) xm = lo;
+                if (lane == 31) xp = hi;
+            }
+            y[r] = fma(a[r], x[r], fma(bl[r], xm, br[r] * xp));
+        }
+    }
+    // v <- e^{-i T tau} v; false (v unchanged) when T is not finite or absurdly
+    // large.  unit: v is e_1 (or any real vector), whose first sub-step needs
+    // real products only.
+    __device__ __forceinline__ bool advance(double tau, double2 (&v)[R], int lane, bool unit) const {
+        const double want = g * fabs(tau);
+        if (!(2.0 * want <= (double)kMaxSub)) return false;
+        const int nsub = max(1, (int)ceil(want));
+        const double h = tau / nsub;
+        int sub = 0;
+        if (unit) {
+            double term[R], y[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) term[r] = v[r].x;
+#pragma unroll 1
+            for (int n = 0; n < kTaylorTerms; ++n) {
+                const double f = h * c_taylor[n];
+                apply(term, y, lane);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    term[r] = f * y[r];  // (-i)^(n+1) comes with the sum
+                    if ((n & 3) == 0) v[r].y -= term[r];
+                    else if ((n & 3) == 1) v[r].x -= term[r];
+                    else if ((n & 3) == 2) v[r].y += term[r];
+                    else v[r].x += term[r];
+                }
+            }
+            sub = 1;
+        }
+        for (; sub < nsub; ++sub) {
+            double2 term[R], sum[R], y[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) term[r] = sum[r] = v[r];
+            // rolled: unrolled, its instructions are fetched from L2 on every use
+#pragma unroll 1
+            for (int n = 0; n < kTaylorTerms; ++n) {
+                const double f = h * c_taylor[n];
+                apply(term, y, lane);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    term[r] = make_double2(f * y[r].y, -f * y[r].x);  // (-i h / n) T term
+                    sum[r].x += term[r].x;
+                    sum[r].y += term[r].y;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = sum[r];
+        }
+        return true;
+    }
+};
 
 // Sum of n partials and the largest of their exponents, in a fixed order, for
 // every thread of the block (every block of a launch gets the same bits).

@@ -102,6 +102,11 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
             slot[b] = cur[D.mode];
         }
     }
+    {
+        std::vector<int> cl;
+        small_plan(cols, M, schedule, cl);
+        for (int b = 0; b < K.B; ++b) K.hdesc[b].small = cl[b];
+    }
     np = 0;
     for (int b = 0; b < K.B; ++b) {
         ColDesc& D = K.hdesc[b];
@@ -174,6 +179,13 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
         ow += (size_t)D.d;
         op += (size_t)D.nblk_max * kPart;
     }
+    {
+        const int rc = small_alloc(K, cols);
+        if (rc != KG_OK) {
+            krylov_free(K);
+            return rc;
+        }
+    }
     KG_TRY(need(cudaMemcpy(K.secs, K.hsec.data(), sizeof(SecView) * K.B, cudaMemcpyHostToDevice), "upload"));
     KG_TRY(need(cudaMemcpy(K.desc, K.hdesc.data(), sizeof(ColDesc) * K.B, cudaMemcpyHostToDevice), "upload"));
     return KG_OK;
@@ -191,6 +203,7 @@ int krylov_set_diag(Krylov& K, const double* diag) {
 }
 
 void krylov_free(Krylov& K) {
+    small_free(K);
     for (auto& kv : K.lists) cudaFree(kv.second.first);
     cudaFree(K.Vbuf);
     cudaFree(K.Sbuf);
@@ -767,8 +780,6 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
 // vector): its error, < 2^-23 |h_k| |v_k[i]| < 1.2e-17 |v_k[i]|, is far
 // below the FP64 rounding of the result, and the FP32 pipe is 64 times wider
 // than the FP64 pipe on this GPU.  Larger coefficients use FP64.
-constexpr double kSmallCoef = 1e-10;
-
 // h_k = s_k <V_k, u> from the exact integer totals of the dots (units 2^26 of
 // 2^(E_k - 1074) 2^(E_u - 1074), E_k the exponent of V_k's image; `keep`: also
 // store E_k, which the dots changed if they re-made the image).
@@ -1176,37 +1187,9 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_tridiag(const ColDesc* desc,
 }
 
 // ------------------------------------ step exponential by a Taylor series
-// c = beta0 e^{-i T tau} e_1 (times s_k per component), the vector of
-// Eq. (udelta), without the eigen-decomposition: the series in (-i T h)
-// with h = tau / n_sub and n_sub chosen so that |T h| <= 1/2 (Gershgorin
-// bound), 18 terms per sub-step (remainder below 1e-22 of the sum).  One
-// warp per column; lane l holds components l and l + 32 (R = 2), so every
-// FP64 instruction serves the whole vector -- the eigen-decomposition's
-// bulge chase is serial.  Modes 0 and 2 as in k_tridiag.
-constexpr int kTaylorTerms = 18;
+// c = beta0 e^{-i T tau} e_1 (times s_k per component) by Tridiag::advance, one
+// warp per column.  Modes 0 and 2 as in k_tridiag.
 constexpr int kMaxTaus = 32;  // times per column in one mode-2 launch
-
-template <int R>
-__device__ __forceinline__ void tri_apply(const double (&a)[R], const double (&bl)[R], const double (&br)[R],
-                                          const double2 (&x)[R], double2 (&y)[R], int lane) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        // x_{k-1} and x_{k+1} for k = lane + 32 r
-        double2 xm, xp;
-        xm.x = __shfl_up_sync(0xffffffffu, x[r].x, 1);
-        xm.y = __shfl_up_sync(0xffffffffu, x[r].y, 1);
-        xp.x = __shfl_down_sync(0xffffffffu, x[r].x, 1);
-        xp.y = __shfl_down_sync(0xffffffffu, x[r].y, 1);
-        const double2 lo = r > 0 ? x[r > 0 ? r - 1 : 0] : make_double2(0.0, 0.0);
-        const double2 hi = r + 1 < R ? x[r + 1 < R ? r + 1 : r] : make_double2(0.0, 0.0);
-        const double lox = __shfl_sync(0xffffffffu, lo.x, 31), loy = __shfl_sync(0xffffffffu, lo.y, 31);
-        const double hix = __shfl_sync(0xffffffffu, hi.x, 0), hiy = __shfl_sync(0xffffffffu, hi.y, 0);
-        if (lane == 0) xm = make_double2(lox, loy);
-        if (lane == 31) xp = make_double2(hix, hiy);
-        y[r].x = fma(a[r], x[r].x, fma(bl[r], xm.x, br[r] * xp.x));
-        y[r].y = fma(a[r], x[r].y, fma(bl[r], xm.y, br[r] * xp.y));
-    }
-}
 
 template <int R>
 __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, ColScalars* cs, int B, int Mcap,
@@ -1223,18 +1206,8 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, Co
                 for (int k = lane; k < Mcap; k += 32) cq[((size_t)b * ntau + t) * Mcap + k] = make_double2(0.0, 0.0);
         return;
     }
-    double a[R], bl[R], br[R];
-    double g = 0.0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int k = lane + 32 * r;
-        a[r] = k < m ? C->alpha[k] : 0.0;
-        bl[r] = (k < m && k >= 1) ? C->beta[k] : 0.0;      // couples k-1 and k
-        br[r] = (k + 1 < m) ? C->beta[k + 1] : 0.0;         // couples k and k+1
-        g = fmax(g, fabs(a[r]) + fabs(bl[r]) + fabs(br[r]));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
+    Tridiag<R> T;
+    T.load(C->alpha, C->beta, m, lane);
     const double beta0 = C->beta0;
     const int nt = mode == 0 ? 1 : ntau;
     // Several times of one sign (mode 2: quadrature nodes) are taken in order
@@ -1267,33 +1240,13 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, Co
         tprev = tfull;
         // a non-finite or absurdly large T (more than kMaxSub sub-steps)
         // cannot be exponentiated this way: report it instead of looping
-        const double want = 2.0 * g * fabs(tau);
-        if (!(want <= (double)kMaxSub)) {
+        if (!T.advance(tau, v, lane, tau == tfull)) {
             if (lane == 0) C->status = KG_ENUMERIC;
             for (int k = lane; k < Mcap; k += 32) C->c[k] = make_double2(0.0, 0.0);
             if (mode == 2)
                 for (int t2 = 0; t2 < ntau; ++t2)
                     for (int k = lane; k < Mcap; k += 32) cq[((size_t)b * ntau + t2) * Mcap + k] = make_double2(0.0, 0.0);
             return;
-        }
-        const int nsub = max(1, (int)ceil(want));
-        const double h = tau / nsub;
-        for (int sub = 0; sub < nsub; ++sub) {
-            double2 term[R], sum[R], y[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) term[r] = sum[r] = v[r];
-            for (int n = 1; n <= kTaylorTerms; ++n) {
-                tri_apply<R>(a, bl, br, term, y, lane);
-                const double f = h / n;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    term[r] = make_double2(f * y[r].y, -f * y[r].x);  // (-i h / n) T term
-                    sum[r].x += term[r].x;
-                    sum[r].y += term[r].y;
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = sum[r];
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -1345,7 +1298,7 @@ int launch_tridiag(Krylov& K, int mode, cudaStream_t st) {
 // Re = T1 - T2, Im = T3 - T1 - T2), or four without it.
 template <int NOV>
 __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const int4* items, ColScalars* cs,
-                                                      unsigned* cnt) {
+                                                      unsigned* cnt, int fused) {
     __shared__ double2 coef[kMaxMgs];
     __shared__ double csum[kMaxMgs];
     __shared__ int idx64[kMaxMgs], idx32[kMaxMgs];
@@ -1355,6 +1308,9 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
     __shared__ double bs[2 * NOV + 2], red[2 * NOV + 2];
     KG_ITEM();
     const int m = C->m_eff;
+    // a space from kg_small.cu comes without the planes
+    const double* Sb = fused ? nullptr : D.S;
+    const float2* V32 = fused ? nullptr : D.V32;
     if (threadIdx.x < 32) {  // the first warp sorts the terms, one per lane
         const int lane = threadIdx.x;
         double cmax = 0.0;
@@ -1370,7 +1326,7 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
             const int k = k0 + lane;
             const double2 c = k < m ? C->c[k] : make_double2(0.0, 0.0);
             const double sk = k < m ? C->scale[k] : 0.0;
-            const bool small = D.V32 && sk > 0.0 && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
+            const bool small = V32 && sk > 0.0 && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
             const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, k < m && small);
             const unsigned before = (1u << lane) - 1u;
             if (k < m && small) {
@@ -1400,8 +1356,6 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
     double acc[2 * NOV + 2];
 #pragma unroll
     for (int k = 0; k < 2 * NOV + 2; ++k) acc[k] = 0.0;
-    const double* Sb = D.S;
-    const float2* V32 = D.V32;
     KG_FOR(i) {
         double2 u;
         if (Sb) {
@@ -1482,10 +1436,10 @@ int launch_combine(Krylov& K, cudaStream_t st) {
     ProfScope ps("combine", st);
     const int4* items;
     int n;
-#define KG_COMB(NOV)                                                              \
-    do {                                                                          \
-        KG_TRY(work_list(K, (const void*)k_combine<NOV>, -1, &items, &n));        \
-        k_combine<NOV><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, K.cnt);       \
+#define KG_COMB(NOV)                                                                                        \
+    do {                                                                                                    \
+        KG_TRY(work_list(K, (const void*)k_combine<NOV>, -1, &items, &n)); \
+        k_combine<NOV><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, K.cnt, K.fused ? 1 : 0);                \
     } while (0)
     if (n_ov == 0) KG_COMB(0);
     else if (n_ov <= 4) KG_COMB(4);
@@ -1562,6 +1516,8 @@ int launch_set_slots(Krylov& K, int value, cudaStream_t st) {
 int prepare_step(Krylov& K, int reorth) {
     const int4* items;
     int n;
+    K.fused = small_steps(K, reorth);
+    if (K.fused) return KG_OK;
     KG_TRY(prepare_hpsi_lists(K));
     KG_TRY(work_list(K, (const void*)k_colnorm, -1, &items, &n));
     KG_TRY(work_list(K, (const void*)k_update, -1, &items, &n));
@@ -1583,6 +1539,8 @@ int prepare_step(Krylov& K, int reorth) {
 
 // Lanczos space of every column's V_0.
 int build_space(Krylov& K, int reorth, cudaStream_t st) {
+    K.fused = small_steps(K, reorth);
+    if (K.fused) return launch_small(K, false, st);
     KG_TRY(launch_colnorm(K, st));
     for (int j = 0; j < K.M; ++j) {
         KG_TRY(launch_lanczos_hpsi(K, j, st));
@@ -1601,10 +1559,13 @@ int build_space(Krylov& K, int reorth, cudaStream_t st) {
 }
 
 int enqueue_step(Krylov& K, int reorth, cudaStream_t st) {
+    if (small_steps(K, reorth)) {
+        K.fused = true;
+        return launch_small(K, true, st);
+    }
     KG_TRY(build_space(K, reorth, st));
     KG_TRY(launch_tridiag(K, 0, st));
-    KG_TRY(launch_combine(K, st));
-    return KG_OK;
+    return launch_combine(K, st);
 }
 
 int column_rc(int status, const char* what) {
