@@ -309,6 +309,7 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
             for (int k = threadIdx.x; k < n; k += blockDim.x) amp[k] = ha[k];
         }
     }
+    chain_wait();
     const bool writer = blk == 0 && threadIdx.x == 0;
     NormHead H;
     if (j > 0) {
@@ -365,6 +366,7 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
         acc = fma(xv.x, r.x, fma(xv.y, r.y, acc));  // Re conj(x) r
         ew = max(ew, max(exp_field(r.x), exp_field(r.y)));
     }
+    chain_next();
     block_partial(sj * acc, ew, sh.sm, sh.smi, D.part_a + blk);
     if (writer) C->n_alpha = nblk;
 }
@@ -446,13 +448,9 @@ int launch_lanczos_hpsi(Krylov& K, int j, cudaStream_t st) {
         // one launch per group of columns whose gathered vectors fit in L2
         for (int g = 0; g < K.ngroups[mode]; ++g) {
             KG_TRY(work_list(K, kern, mode, &items, &n, g));
-            switch (mode) {
-                case 3: k_lanczos_hpsi<3><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
-                case 0: k_lanczos_hpsi<0><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
-                case 1: k_lanczos_hpsi<1><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
-                default: k_lanczos_hpsi<2><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j); break;
-            }
-            KG_LAUNCHED();
+            const auto k = mode == 3 ? &k_lanczos_hpsi<3> : mode == 0 ? &k_lanczos_hpsi<0> : mode == 1 ? &k_lanczos_hpsi<1>
+                                                                                                       : &k_lanczos_hpsi<2>;
+            KG_TRY(launch_chained(k, n, kThreads, 0, st, K.desc, items, K.cs, j));
         }
     }
     return KG_OK;

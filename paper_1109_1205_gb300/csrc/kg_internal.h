@@ -394,6 +394,40 @@ const char* last_error();
 #ifdef __CUDACC__
 namespace kg {
 
+// Programmatic dependent launch.  The phases of a Lanczos step are short
+// kernels in one stream, each reading what the one before wrote.  A kernel
+// launched by launch_chained may start while its predecessor runs; it reads
+// only its work list and descriptors (constant during a step) before
+// chain_wait, which returns when the predecessor has completed and its writes
+// are visible.  chain_next lets the successor start; it stands at the end of
+// the streaming loops, because blocks that start earlier settle on the first
+// SMs with room and leave a one-wave grid uneven (an impulse at the start of
+// every kernel cost 3 to 6%).  At the end it gains 2.5% on one column of
+// 853,776 states (14.42 -> 14.06 ms for five steps), 4% on 96 columns of up to
+// 52,920 states (191 -> 183 ms for 60 steps).
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+int launch_chained(void (*kern)(P...), int blocks, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    if (e != cudaSuccess) return cuda_fail(e, "kernel launch", __FILE__, __LINE__);
+    count_launch();
+    return KG_OK;
+}
+
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }

@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(kThreads) k_colnorm(const ColDesc* desc, const
     __shared__ int smi[kThreads / 32];
     __shared__ double bs[2], red[2];
     KG_ITEM();
+    chain_wait();
     const double2* x = D.V;
     double acc[1] = {0.0};
     int em = 0;
@@ -321,9 +322,7 @@ int launch_colnorm(Krylov& K, cudaStream_t st) {
     const int4* items;
     int n;
     KG_TRY(work_list(K, (const void*)k_colnorm, -1, &items, &n));
-    k_colnorm<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, K.M, K.cnt);
-    KG_LAUNCHED();
-    return KG_OK;
+    return launch_chained(k_colnorm, n, kThreads, 0, st, K.desc, items, K.cs, K.M, K.cnt);
 }
 
 // ---------------------------------------- Gram-Schmidt coefficients
@@ -546,14 +545,6 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
     int4* const ua = reinterpret_cast<int4*>(dyn + S * P::kStage);  // [2][kThreads] image of u
     int2* const ub = reinterpret_cast<int2*>(dyn + S * P::kStage + 2 * kThreads * 16);
     KG_ITEM();
-    if (j >= C->m_eff) return;
-    const int d = D.d;
-    // this block's elements [e0, e0 + len), in tiles of T
-    const int run = (int)(((long long)d + nblk - 1) / nblk);
-    const size_t e0 = (size_t)min((long long)d, (long long)blk * run);
-    const int len = (int)min((long long)run, (long long)d - (long long)e0);
-    const int nt = (len + T - 1) / T, nr = (len + kThreads - 1) / kThreads;
-    const int4* Ib = D.I + (size_t)k0 * d + e0;
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int q = 0; q < S; ++q) {
@@ -562,7 +553,16 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
         }
         mbar_init_fence();
     }
-    __syncthreads();
+    chain_wait();
+    if (j >= C->m_eff) return;
+    const int d = D.d;
+    // this block's elements [e0, e0 + len), in tiles of T
+    const int run = (int)(((long long)d + nblk - 1) / nblk);
+    const size_t e0 = (size_t)min((long long)d, (long long)blk * run);
+    const int len = (int)min((long long)run, (long long)d - (long long)e0);
+    const int nt = (len + T - 1) / T, nr = (len + kThreads - 1) / kThreads;
+    const int4* Ib = D.I + (size_t)k0 * d + e0;
+    __syncthreads();  // the stages' barriers are ready
     const int lane = threadIdx.x & 31;
     const bool copies = threadIdx.x >= P::compute;
     auto issue = [&](int t) {  // by the copying warp: tile t into its stage
@@ -693,6 +693,7 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
         if (r + 1 < nr) form_u(r + 1);
         block_bar(1, P::compute);
     }
+    chain_next();
     flush();
     if (!ok) C->status = KG_ETIMEOUT;
 }
@@ -754,9 +755,7 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
         const int4* items;
         int n;
         KG_TRY(work_list(K, (const void*)ik.kern, -1, &items, &n, -1, ik.threads, ik.smem, kDotMinRun));
-        ik.kern<<<n, ik.threads, ik.smem, st>>>(K.desc, items, K.cs, j, k0);
-        KG_LAUNCHED();
-        return KG_OK;
+        return launch_chained(ik.kern, n, ik.threads, ik.smem, st, K.desc, items, K.cs, j, k0);
     }
     const DotsKernel kern = dots_kernel(nk);
     const int4* items;
@@ -812,6 +811,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     __shared__ int smi[kThreads / 32];
     __shared__ Partial pair[kThreads / 32];
     KG_ITEM();
+    chain_wait();
     if (j >= C->m_eff) return;
     const bool writer = blk == 0 && threadIdx.x == 0;
     const int d = D.d;
@@ -983,6 +983,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     } else {
         KG_FOR(i) element(i);
     }
+    chain_next();
     block_partial(acc, em, sm, smi, D.part_n + blk);
     if (writer) {
         C->n_norm = nblk;
@@ -998,14 +999,13 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
 __global__ void __launch_bounds__(kThreads) k_resolve(const ColDesc* desc, ColScalars* cs, int j) {
     __shared__ Partial pair[kThreads / 32];
     const ColDesc D = desc[blockIdx.x];
+    chain_wait();
     resolve_norm(D, cs + blockIdx.x, j, threadIdx.x == 0, pair);
 }
 
 int launch_resolve(Krylov& K, int j, cudaStream_t st) {
     ProfScope ps("resolve", st);
-    k_resolve<<<K.B, kThreads, 0, st>>>(K.desc, K.cs, j);
-    KG_LAUNCHED();
-    return KG_OK;
+    return launch_chained(k_resolve, K.B, kThreads, 0, st, K.desc, K.cs, j);
 }
 
 int launch_update(Krylov& K, int j, int level, bool second, cudaStream_t st) {
@@ -1014,9 +1014,7 @@ int launch_update(Krylov& K, int j, int level, bool second, cudaStream_t st) {
     int n;
     KG_TRY(work_list(K, (const void*)k_update, -1, &items, &n));
     const int exact = level >= 1 && use_int_dots(K, second);
-    k_update<<<n, kThreads, 0, st>>>(K.desc, items, K.cs, j, level, second ? 1 : 0, exact);
-    KG_LAUNCHED();
-    return KG_OK;
+    return launch_chained(k_update, n, kThreads, 0, st, K.desc, items, K.cs, j, level, second ? 1 : 0, exact);
 }
 
 // ------------------------------------------- tridiagonal eigenproblem
@@ -1196,6 +1194,7 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, Co
                                                         int mode, const double* taus, int ntau, double2* cq) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x * kTriWarps + warp;
+    chain_wait();
     if (b >= B) return;
     ColScalars* C = cs + b;
     const int m = C->m_eff;
@@ -1267,12 +1266,8 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, Co
 
 static int launch_texp(Krylov& K, int mode, const double* taus, int ntau, double2* cq, cudaStream_t st) {
     const int nb = (K.B + kTriWarps - 1) / kTriWarps;
-    if (K.M <= 32)
-        k_texp<1><<<nb, 32 * kTriWarps, 0, st>>>(K.desc, K.cs, K.B, K.M, mode, taus, ntau, cq);
-    else
-        k_texp<2><<<nb, 32 * kTriWarps, 0, st>>>(K.desc, K.cs, K.B, K.M, mode, taus, ntau, cq);
-    KG_LAUNCHED();
-    return KG_OK;
+    return launch_chained(K.M <= 32 ? &k_texp<1> : &k_texp<2>, nb, 32 * kTriWarps, 0, st, K.desc, K.cs, K.B, K.M, mode,
+                          taus, ntau, cq);
 }
 
 int launch_tridiag(Krylov& K, int mode, cudaStream_t st) {
@@ -1307,6 +1302,7 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
     __shared__ double sm[(kThreads / 32) * (2 * NOV + 2)];
     __shared__ double bs[2 * NOV + 2], red[2 * NOV + 2];
     KG_ITEM();
+    chain_wait();
     const int m = C->m_eff;
     // a space from kg_small.cu comes without the planes
     const double* Sb = fused ? nullptr : D.S;
@@ -1436,18 +1432,9 @@ int launch_combine(Krylov& K, cudaStream_t st) {
     ProfScope ps("combine", st);
     const int4* items;
     int n;
-#define KG_COMB(NOV)                                                                                        \
-    do {                                                                                                    \
-        KG_TRY(work_list(K, (const void*)k_combine<NOV>, -1, &items, &n)); \
-        k_combine<NOV><<<n, kThreads, 0, st>>>(K.desc, items, K.cs, K.cnt, K.fused ? 1 : 0);                \
-    } while (0)
-    if (n_ov == 0) KG_COMB(0);
-    else if (n_ov <= 4) KG_COMB(4);
-    else if (n_ov <= 12) KG_COMB(12);
-    else KG_COMB(32);
-#undef KG_COMB
-    KG_LAUNCHED();
-    return KG_OK;
+    const auto kern = n_ov == 0 ? &k_combine<0> : n_ov <= 4 ? &k_combine<4> : n_ov <= 12 ? &k_combine<12> : &k_combine<32>;
+    KG_TRY(work_list(K, (const void*)kern, -1, &items, &n));
+    return launch_chained(kern, n, kThreads, 0, st, K.desc, items, K.cs, K.cnt, K.fused ? 1 : 0);
 }
 
 // -------------------------------------------- ground-state residual
