@@ -100,3 +100,16 @@ def test_small_columns_in_one_batch(large):
     for i, m in enumerate(models):
         ref = kg.Sector(m).green_equilibrium([(0, 0), (0, 1)], 0.05, 12, kg.kg_opts_default(schedule=4))
         assert np.max(np.abs(gg[i] - ref[0])) < TOL and np.max(np.abs(gl[i] - ref[1])) < TOL
+
+
+@pytest.mark.parametrize("M_gs", [2, 3, 33, 64, 100, 255])
+def test_lowest_ritz_pair(M_gs):
+    """Ground states from restarts of every length class, against the oracle:
+    energy 1e-12 relative, the vector to 1e-10 in overlap (its residual is
+    1e-12 and the gap above 0.1)."""
+    for m in (W.random_model(6, 3, 2, seed=9), W.siam_chain(7, 3.0, 3, 4, field=0.3)):
+        s = kg.Sector(m)
+        e, res, gap = s.ground_state(kg.kg_opts_default(M_gs=M_gs, max_restarts=4000, tol_resid=1e-11))
+        e_ref, psi, _ = oracle.Sector(m).ground_state()
+        assert abs(e - e_ref) < 1e-12 * max(1.0, abs(e_ref)) and gap > 0.0
+        assert abs(abs(np.vdot(psi, s.ground_state_vector())) - 1.0) < 1e-10
