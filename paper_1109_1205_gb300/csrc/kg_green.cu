@@ -442,111 +442,234 @@ int green_equilibrium_batched(kg_sector* const* s, int n_inst, const int* orb, i
 }
 
 // --------------------------------------------------- Gram, step (iv)
-// G[p][q] = <X_p | X_q> for the upper-triangle tiles (p tile <= q tile) of a
-// set of nv vectors of dimension d, FP64 on the CUDA cores.  32 x 32 output
-// tile per block, 2 x 2 complex outputs per thread, 16-element slabs of the
-// vectors staged in shared memory, split over d by gridDim.z (partials).
-constexpr int kGT = 32, kGK = 16;
+// G[p][q] = <X_p | X_q> of nv vectors of dimension d, upper-triangle 32 x 32
+// tiles, the lower triangle by Hermiticity.
+//
+// A complex product costs four FP64 multiply-adds, two SM cycles for a lane on
+// this GPU, or sixteen 32 x 32 -> 64 bit integer ones of 52-bit fixed-point
+// images (kg_krylov.cu, the exact dots), half a cycle.  So the vectors are
+// converted on their own largest exponents when a tile is staged, the products
+// are summed exactly and go to FP64 every kGramFlush elements.  The images'
+// rounding, 2^-53 of a vector's largest component per element, adds at most
+// 2^-53 ||x|| ||y|| to a sum, less than the rounding of an FP64 sum.
+//
+// A thread takes 2 x 2 outputs {I, I + H} x {J, J + H} of a tile, H half its
+// rows, so that neighbouring lanes read neighbouring rows; a diagonal tile
+// keeps I <= J only, and the threads in use are packed into the first warps
+// (the multiply-add pipe is what bounds this kernel, so idle warps cost
+// nothing).  The vectors are split over gridDim.y slabs, at least eight staged
+// steps each.  48 vectors of 731,808 states: 21.8 ms in FP64 with one slab per
+// 4,096 states and whole diagonal tiles, 5 ms now; 12 vectors 1.05 -> 0.55 ms;
+// 10 vectors of 3,920 states 4.0 -> 0.06 ms.
+constexpr int kGT = 32, kGK = 16, kGramFlush = 256;
 
-__global__ void __launch_bounds__(256) k_gram(const double2* __restrict__ X, int nv, int d, int ntile,
-                                              const int2* __restrict__ tiles, double2* __restrict__ part) {
-    __shared__ double2 As[kGT][kGK + 1];
-    __shared__ double2 Bs[kGK][kGT + 1];
-    const int2 tl = tiles[blockIdx.x];
-    const int p0 = tl.x * kGT, q0 = tl.y * kGT;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int z = blockIdx.y, nz = gridDim.y;
-    const int slab = (d + nz - 1) / nz;
-    const int i_begin = z * slab, i_end = min(d, i_begin + slab);
-    double2 acc[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
-    for (int i0 = i_begin; i0 < i_end; i0 += kGK) {
-        // 32 rows x 16 elements of each operand: 2 loads per thread
-        for (int t = threadIdx.x; t < kGT * kGK; t += 256) {
-            const int r = t / kGK, c = t % kGK;
-            const int i = i0 + c;
-            const int p = p0 + r, q = q0 + r;
-            As[r][c] = (p < nv && i < i_end) ? X[(size_t)p * d + i] : make_double2(0.0, 0.0);
-            Bs[c][r] = (q < nv && i < i_end) ? X[(size_t)q * d + i] : make_double2(0.0, 0.0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int c = 0; c < kGK; ++c) {
-            const double2 a0 = As[ty][c], a1 = As[ty + 16][c];
-            const double2 b0 = Bs[c][tx], b1 = Bs[c][tx + 16];
-            acc[0][0].x = fma(a0.x, b0.x, fma(a0.y, b0.y, acc[0][0].x));
-            acc[0][0].y = fma(a0.x, b0.y, fma(-a0.y, b0.x, acc[0][0].y));
-            acc[0][1].x = fma(a0.x, b1.x, fma(a0.y, b1.y, acc[0][1].x));
-            acc[0][1].y = fma(a0.x, b1.y, fma(-a0.y, b1.x, acc[0][1].y));
-            acc[1][0].x = fma(a1.x, b0.x, fma(a1.y, b0.y, acc[1][0].x));
-            acc[1][0].y = fma(a1.x, b0.y, fma(-a1.y, b0.x, acc[1][0].y));
-            acc[1][1].x = fma(a1.x, b1.x, fma(a1.y, b1.y, acc[1][1].x));
-            acc[1][1].y = fma(a1.x, b1.y, fma(-a1.y, b1.x, acc[1][1].y));
-        }
-        __syncthreads();
+// Largest exponent field of each vector (emax pre-set to 0).
+__global__ void __launch_bounds__(kThreads) k_gram_exp(const double2* __restrict__ X, int d, int* emax) {
+    __shared__ int sm[kThreads / 32];
+    const double2* x = X + (size_t)blockIdx.y * d;
+    int m = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d; i += gridDim.x * blockDim.x) {
+        const double2 v = x[i];
+        m = max(m, max(exp_field(v.x), exp_field(v.y)));
     }
-    double2* out = part + (size_t)z * ntile * kGT * kGT + (size_t)blockIdx.x * kGT * kGT;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) out[(ty + 16 * a) * kGT + tx + 16 * b] = acc[a][b];
+    m = block_max_int(m, sm);
+    if (threadIdx.x == 0) atomicMax(emax + blockIdx.y, m);
 }
 
-__global__ void k_gram_reduce(const double2* part, int nz, int ntile, const int2* tiles, int nv, double2* G) {
-    const int t = blockIdx.x, e = threadIdx.x + blockDim.x * blockIdx.y;
+__global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, int nv, int d, int ntile, int slab,
+                                                 const int2* __restrict__ tiles, const int* __restrict__ emax,
+                                                 double2* __restrict__ part) {
+    __shared__ int4 st[2][2 * kGT][kGK + 1];  // rows of the two operands, 16-byte stride between rows mod 128
+    const int2 tl = tiles[blockIdx.x];
+    const bool diag = tl.x == tl.y;
+    const int p0 = tl.x * kGT, q0 = tl.y * kGT;
+    const int Hp = (min(kGT, nv - p0) + 1) / 2, Hq = (min(kGT, nv - q0) + 1) / 2;
+    const int i_begin = blockIdx.y * slab, i_end = min(d, i_begin + slab);
+    // this thread's outputs
+    int I = 0, J = 0;
+    const int n_use = diag ? Hp * (Hp + 1) / 2 : Hp * Hq;
+    const bool use = (int)threadIdx.x < n_use;
+    if (use) {
+        int t = threadIdx.x;
+        if (diag) {
+            while (t >= Hp - I) t -= Hp - I++;
+            J = I + t;
+        } else {
+            I = t / Hq;
+            J = t - I * Hq;
+        }
+    }
+    const int rows = diag ? kGT : 2 * kGT;
+    // staging: four elements per thread (two for a diagonal tile), one step ahead
+    const int c = threadIdx.x & (kGK - 1), r0 = threadIdx.x / kGK;  // rows r0, r0 + 16, ...
+    double2 nx[4];
+    int ex[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = r0 + 16 * u, v = r < kGT ? p0 + r : q0 + r - kGT;
+        ex[u] = r < rows && v < nv ? emax[v] : 0;
+    }
+    auto load = [&](int i0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = r0 + 16 * u, v = r < kGT ? p0 + r : q0 + r - kGT, i = i0 + c;
+            nx[u] = r < rows && v < nv && i < i_end ? X[(size_t)v * d + i] : make_double2(0.0, 0.0);
+        }
+    };
+    auto stage = [&](int b) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = r0 + 16 * u;
+            if (r < rows) st[b][r][c] = fix_image(nx[u], ex[u]);
+        }
+    };
+    double2 acc[2][2];
+    long long re[2][2][3], im[2][2][3];
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            acc[x][y] = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) re[x][y][q] = im[x][y][q] = 0;
+        }
+    auto flush = [&]() {
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const long long rl = re[x][y][1] + (re[x][y][2] >> 26), il = im[x][y][1] + (im[x][y][2] >> 26);
+                acc[x][y].x += fma((double)rl, 0x1p-26, (double)re[x][y][0]);
+                acc[x][y].y += fma((double)il, 0x1p-26, (double)im[x][y][0]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) re[x][y][q] = im[x][y][q] = 0;
+            }
+    };
+    load(i_begin);
+    stage(0);
+    __syncthreads();
+    int held = 0;
+    for (int i0 = i_begin, b = 0; i0 < i_end; i0 += kGK, b ^= 1) {
+        if (i0 + kGK < i_end) load(i0 + kGK);
+        if (use) {
+            const int4* A = &st[b][I][0];
+            const int4* B = &st[b][(diag ? 0 : kGT) + J][0];
+            const int ah = Hp * (kGK + 1), bh = Hq * (kGK + 1);
+#pragma unroll 2
+            for (int k = 0; k < kGK; ++k) {
+                const int4 a0 = A[k], a1 = A[ah + k], b0 = B[k], b1 = B[bh + k];
+                const int2 m0 = make_int2(-b0.x, -b0.y), m1 = make_int2(-b1.x, -b1.y);
+                cdot_fix(a0, b0, m0, re[0][0], im[0][0]);
+                cdot_fix(a0, b1, m1, re[0][1], im[0][1]);
+                cdot_fix(a1, b0, m0, re[1][0], im[1][0]);
+                cdot_fix(a1, b1, m1, re[1][1], im[1][1]);
+            }
+            held += kGK;
+            if (held == kGramFlush) {
+                flush();
+                held = 0;
+            }
+        }
+        if (i0 + kGK < i_end) stage(b ^ 1);
+        __syncthreads();
+    }
+    if (!use) return;
+    flush();
+    double2* out = part + ((size_t)blockIdx.y * ntile + blockIdx.x) * kGT * kGT;
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) out[(I + x * Hp) * kGT + J + y * Hq] = acc[x][y];
+}
+
+__global__ void k_gram_reduce(const double2* part, int nz, int ntile, const int2* tiles, const int* emax, int nv,
+                              double2* G) {
+    const int e = threadIdx.x + blockDim.x * blockIdx.y;
     if (e >= kGT * kGT) return;
+    const int2 tl = tiles[blockIdx.x];
+    const bool diag = tl.x == tl.y;
+    const int Hp = (min(kGT, nv - tl.x * kGT) + 1) / 2, Hq = (min(kGT, nv - tl.y * kGT) + 1) / 2;
+    const int r = e / kGT, c = e % kGT, p = tl.x * kGT + r, q = tl.y * kGT + c;
+    if (r >= 2 * Hp || c >= 2 * Hq || p >= nv || q >= nv) return;
+    if (diag && r % Hp > c % Hp) return;         // not computed
+    if (diag && r == c + Hp) return;             // its mirror is
     double2 s = make_double2(0.0, 0.0);
     for (int z = 0; z < nz; ++z) {
-        const double2 v = part[((size_t)z * ntile + t) * kGT * kGT + e];
+        const double2 v = part[((size_t)z * ntile + blockIdx.x) * kGT * kGT + e];
         s.x += v.x;
         s.y += v.y;
     }
-    const int2 tl = tiles[t];
-    const int p = tl.x * kGT + e / kGT, q = tl.y * kGT + e % kGT;
-    if (p < nv && q < nv) G[(size_t)p * nv + q] = s;
+    // units of the images; a non-finite vector has none
+    const double f = emax[p] == 2047 || emax[q] == 2047 ? nan("") : ldexp(1.0, emax[p] + emax[q] - 2096);
+    s.x *= f;
+    s.y = p == q ? 0.0 * f : s.y * f;
+    G[(size_t)p * nv + q] = s;
+    G[(size_t)q * nv + p] = make_double2(s.x, -s.y);
 }
+
+// Tiles, slabs and scratch of one Gram matrix on the device.
+struct GramPlan {
+    int nv = 0, ntile = 0, nz = 1, slab = 0;
+    int2* tiles = nullptr;
+    double2* part = nullptr;
+    int* emax = nullptr;
+    int init(int nv_, int d, int nsm) {
+        nv = nv_;
+        const int nt = (nv + kGT - 1) / kGT;
+        std::vector<int2> v;
+        for (int a = 0; a < nt; ++a)
+            for (int b = a; b < nt; ++b) v.push_back(make_int2(a, b));
+        ntile = (int)v.size();
+        // four blocks per SM, but no fewer than 8 staged steps each
+        nz = std::max(1, std::min((nsm * 4 + ntile - 1) / ntile, (d + 8 * kGK - 1) / (8 * kGK)));
+        slab = ((d + nz - 1) / nz + kGK - 1) / kGK * kGK;
+        nz = std::max(1, (d + slab - 1) / slab);
+        if (cudaMalloc(&tiles, sizeof(int2) * ntile) != cudaSuccess ||
+            cudaMalloc(&part, sizeof(double2) * (size_t)nz * ntile * kGT * kGT) != cudaSuccess ||
+            cudaMalloc(&emax, sizeof(int) * nv) != cudaSuccess) {
+            cudaGetLastError();
+            release();
+            set_error("Gram scratch of %d vectors", nv);
+            return KG_ENOMEM;
+        }
+        KG_CUDA(cudaMemcpy(tiles, v.data(), sizeof(int2) * ntile, cudaMemcpyHostToDevice));
+        return KG_OK;
+    }
+    int run(const double2* X, int d, int nsm, double2* G, cudaStream_t st) const {
+        ProfScope ps("gram", st);
+        KG_CUDA(cudaMemsetAsync(emax, 0, sizeof(int) * nv, st));
+        const int be = std::max(1, std::min((d + kThreads - 1) / kThreads, (nsm * 8 + nv - 1) / nv));
+        k_gram_exp<<<dim3(be, nv), kThreads, 0, st>>>(X, d, emax);
+        k_gram<<<dim3(ntile, nz), 256, 0, st>>>(X, nv, d, ntile, slab, tiles, emax, part);
+        k_gram_reduce<<<dim3(ntile, kGT * kGT / 256), 256, 0, st>>>(part, nz, ntile, tiles, emax, nv, G);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "kernel launch", __FILE__, __LINE__);
+        count_launch(3);
+        return KG_OK;
+    }
+    void release() {
+        cudaFree(tiles);
+        cudaFree(part);
+        cudaFree(emax);
+        tiles = nullptr;
+        part = nullptr;
+        emax = nullptr;
+    }
+};
 
 // Full Hermitian Gram matrix (host, nv x nv complex) of the nv vectors X.
 int gram(const double2* X, int nv, int d, int nsm, std::vector<std::complex<double>>& G, cudaStream_t st) {
-    const int nt = (nv + kGT - 1) / kGT;
-    std::vector<int2> tiles;
-    for (int a = 0; a < nt; ++a)
-        for (int b = a; b < nt; ++b) tiles.push_back(make_int2(a, b));
-    const int ntile = (int)tiles.size();
-    int nz = std::max(1, std::min((nsm * 2 + ntile - 1) / ntile, (d + 4095) / 4096));
-    int2* dt = nullptr;
-    double2 *part = nullptr, *dG = nullptr;
-    int rc = KG_OK;
-    if (cudaMalloc(&dt, sizeof(int2) * ntile) != cudaSuccess ||
-        cudaMalloc(&part, sizeof(double2) * (size_t)nz * ntile * kGT * kGT) != cudaSuccess ||
-        cudaMalloc(&dG, sizeof(double2) * (size_t)nv * nv) != cudaSuccess)
-        rc = KG_ENOMEM;
-    if (rc == KG_OK) {
-        cudaMemcpyAsync(dt, tiles.data(), sizeof(int2) * ntile, cudaMemcpyHostToDevice, st);
-        cudaMemsetAsync(dG, 0, sizeof(double2) * (size_t)nv * nv, st);
-        ProfScope ps("gram", st);
-        k_gram<<<dim3(ntile, nz), 256, 0, st>>>(X, nv, d, ntile, dt, part);
-        count_launch();
-        k_gram_reduce<<<dim3(ntile, (kGT * kGT + 255) / 256), 256, 0, st>>>(part, nz, ntile, dt, nv, dG);
-        count_launch();
-        std::vector<double2> h((size_t)nv * nv);
-        if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(h.data(), dG, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            rc = cuda_fail(cudaGetLastError(), "gram", __FILE__, __LINE__);
-        G.assign((size_t)nv * nv, 0.0);
-        for (int p = 0; p < nv; ++p)
-            for (int q = p; q < nv; ++q) {
-                const double2 v = h[(size_t)p * nv + q];
-                G[(size_t)p * nv + q] = std::complex<double>(v.x, v.y);
-                G[(size_t)q * nv + p] = std::complex<double>(v.x, -v.y);
-            }
-    }
-    cudaFree(dt);
-    cudaFree(part);
+    GramPlan P;
+    KG_TRY(P.init(nv, d, nsm));
+    double2* dG = nullptr;
+    int rc = cudaMalloc(&dG, sizeof(double2) * (size_t)nv * nv) == cudaSuccess ? KG_OK : KG_ENOMEM;
+    if (rc == KG_OK) rc = P.run(X, d, nsm, dG, st);
+    G.resize((size_t)nv * nv);
+    if (rc == KG_OK &&
+        (cudaMemcpyAsync(G.data(), dG, sizeof(double2) * G.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+         cudaStreamSynchronize(st) != cudaSuccess))
+        rc = cuda_fail(cudaGetLastError(), "gram", __FILE__, __LINE__);
+    P.release();
     cudaFree(dG);
     return rc;
 }
@@ -1057,6 +1180,7 @@ struct KBlock {
     double2* store = nullptr;  // [slots][na][d_nb]: every row, or only the current one
     int slots = 0;
     double2* ovbuf = nullptr;  // [na][na]
+    kg::GramPlan rowgram;      // of one row's columns
     kg::Krylov K;
     kg::StepRunner R;
     bool ready = false;
@@ -1098,6 +1222,7 @@ static void block_release(KBlock& B) {
     block_release_krylov(B);
     cudaFree(B.store);
     cudaFree(B.ovbuf);
+    B.rowgram.release();
     cudaFree(B.dwork);
     B.store = nullptr;
     B.ovbuf = nullptr;
@@ -1460,7 +1585,8 @@ int keldysh_row(kg_keldysh* X, int k, double* G_les_kk, double* G_gtr_kk) {
         if (rc == KG_OK) rc = block_row(X, B, k, st);
         const int na = (int)B.idx.size(), dn = (int)B.nb->d;
         const double2* xs = B.store + (B.slots > 1 ? (size_t)k * na * dn : 0);
-        if (rc == KG_OK) rc = launch_inner_lib(xs, na, xs, na, dn, B.ovbuf, na, st);
+        if (rc == KG_OK && !B.rowgram.tiles) rc = B.rowgram.init(na, dn, X->fin->nsm);
+        if (rc == KG_OK) rc = B.rowgram.run(xs, dn, X->fin->nsm, B.ovbuf, st);
         std::vector<double2> h((size_t)na * na);
         if (rc == KG_OK &&
             (cudaMemcpyAsync(h.data(), B.ovbuf, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, st) !=
@@ -1475,8 +1601,7 @@ int keldysh_row(kg_keldysh* X, int k, double* G_les_kk, double* G_gtr_kk) {
         if (!G) continue;
         for (int bb = 0; bb < na; ++bb)
             for (int a = 0; a < na; ++a) {
-                // h[bb][a] = <X_a | X_bb>
-                const double2 v = h[(size_t)bb * na + a];
+                const double2 v = h[(size_t)a * na + bb];  // <X_a | X_bb>
                 const std::complex<double> ov(v.x, v.y);
                 int r, c;
                 std::complex<double> g;

@@ -502,22 +502,6 @@ struct IntDots {
 constexpr int kDotFlush = 256;   // elements a thread may add to its 64-bit sums
 constexpr int kDotMinRun = 64;   // fewest elements worth a block
 
-// Re and Im of conj(v) u for v and u given as split 52-bit images (v:
-// {x_hi, x_lo, y_hi, y_lo}; u likewise, m: hi and lo of -Re u), added to sums
-// in units of 2^52 (s[0]), 2^26 (s[1]) and 1 (s[2]) of the full product.
-__device__ __forceinline__ void cdot_fix(const int4 v, const int4 u, const int2 m, long long (&re)[3],
-                                         long long (&im)[3]) {
-    const int p1 = u.x, p0 = u.y, q1 = u.z, q0 = u.w, n1 = m.x, n0 = m.y;
-    // Re = vx ux + vy uy
-    re[0] += (long long)v.x * p1 + (long long)v.z * q1;
-    re[1] += (long long)v.x * p0 + (long long)v.y * p1 + (long long)v.z * q0 + (long long)v.w * q1;
-    re[2] += (long long)v.y * p0 + (long long)v.w * q0;
-    // Im = vx uy - vy ux
-    im[0] += (long long)v.x * q1 + (long long)v.z * n1;
-    im[1] += (long long)v.x * q0 + (long long)v.y * q1 + (long long)v.z * n0 + (long long)v.w * n1;
-    im[2] += (long long)v.y * q0 + (long long)v.w * n0;
-}
-
 // The warp's total of s[0] 2^26 + s[1] + s[2] 2^-26 (|s[0]| < 2^62) as two
 // limbs, total = l1 2^46 + l0.
 __device__ __forceinline__ void warp_limbs(const long long (&s)[3], unsigned long long& l0, unsigned long long& l1) {

@@ -102,6 +102,20 @@ def test_small_columns_in_one_batch(large):
         assert np.max(np.abs(gg[i] - ref[0])) < TOL and np.max(np.abs(gl[i] - ref[1])) < TOL
 
 
+@pytest.mark.parametrize("L,nu,nd", [(3, 1, 2), (5, 2, 2), (7, 3, 3)])
+@pytest.mark.parametrize("n_orb,n_t", [(1, 1), (1, 2), (3, 1), (2, 8), (1, 31), (3, 11), (3, 16), (3, 22)])
+def test_gram_tiles(L, nu, nd, n_orb, n_t):
+    """G(t,t') whose Gram matrices have 1 to 66 vectors (one tile, a ragged
+    second and third one, an odd count) of 3 to 1,225 states.  1e-10 is the bar
+    of the Green's functions; a wrong tile shifts entries of order 0.1."""
+    ini, fin = W.random_model(L, nu, nd, seed=5), W.random_model(L, nu, nd, seed=6)
+    orbs = [(a, 0) for a in range(n_orb)]
+    si, sf = kg.Sector(ini), kg.Sector(fin)
+    gl, gg = kg.kg_green_keldysh(si.handle, sf.handle, orbs, 0.05, n_t)
+    rl, rg = oracle.green_keldysh(ini, fin, orbs, 0.05, n_t)[:2]
+    assert np.max(np.abs(gl - rl)) < 1e-10 and np.max(np.abs(gg - rg)) < 1e-10
+
+
 @pytest.mark.parametrize("M_gs", [2, 3, 33, 64, 100, 255])
 def test_lowest_ritz_pair(M_gs):
     """Ground states from restarts of every length class, against the oracle:
