@@ -283,9 +283,7 @@ __global__ void __launch_bounds__(kThreads) k_hpsi(SecView S, const double2* __r
 // serial tail to every launch.
 struct HpsiShared {
     double2 amp[kMaxL * kMaxL];
-    double sm[kThreads / 32];
-    int smi[kThreads / 32];
-    Partial pair[kThreads / 32];
+    HeadShared head;
     SecView S;
 };
 
@@ -311,19 +309,20 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
     }
     chain_wait();
     const bool writer = blk == 0 && threadIdx.x == 0;
-    NormHead H;
+    HeadShared& H = sh.head;
     if (j > 0) {
-        H = resolve_norm(D, C, j, writer, sh.pair);
+        resolve_norm(D, C, j, writer, H);
     } else {  // the start vector's norm is k_colnorm's
-        H.m_eff = C->m_eff;
-        H.scale = C->scale[0];
-        H.emax = C->emax[0];
-        H.beta = 0.0;
+        if (threadIdx.x == 0) {
+            H.m_eff = C->m_eff;
+            H.scale = C->scale[0];
+            H.emax = C->emax[0];
+            H.cprev = 0.0;
+        }
+        __syncthreads();
     }
     if (j >= H.m_eff) return;
-    __syncthreads();
-    const double sj = H.scale;
-    const double cprev = (j > 0) ? H.beta * C->scale[j - 1] : 0.0;
+    const double sj = H.scale, cprev = H.cprev;
     const int E = (MODE == 3) ? H.emax : 0;
     const double hs = S.h0 * sj;
     // V_j in fixed point, written by the update that produced it (not V_0),
@@ -367,7 +366,7 @@ __device__ __forceinline__ void lanczos_hpsi_item(const ColDesc* desc, ColScalar
         ew = max(ew, max(exp_field(r.x), exp_field(r.y)));
     }
     chain_next();
-    block_partial(sj * acc, ew, sh.sm, sh.smi, D.part_a + blk);
+    block_partial(sj * acc, ew, sh.head.sum, D.part_a + blk);
     if (writer) C->n_alpha = nblk;
 }
 

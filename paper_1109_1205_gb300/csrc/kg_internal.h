@@ -511,32 +511,6 @@ __device__ __forceinline__ int block_max_int(int v, int* sm) {
     return m;
 }
 
-// One block's partial sum and largest exponent, stored in *out.  The warps'
-// sums are added by one warp (a warp's FP64 instruction holds this GPU's FP64
-// pipe for many cycles, so eight serial adds by every thread would cost more
-// than the shuffles).  sm, smi: blockDim / 32 entries.
-__device__ __forceinline__ void block_partial(double v, int e, double* sm, int* smi, Partial* out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum(v);
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) {
-        sm[warp] = v;
-        smi[warp] = e;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < nw ? sm[lane] : 0.0;
-        e = lane < nw ? smi[lane] : 0;
-#pragma unroll
-        for (int o = kThreads / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        e = __reduce_max_sync(0xffffffffu, e);
-        if (lane == 0) {
-            out->v = v;
-            out->e = e;
-        }
-    }
-}
-
 // Biased exponent field of an FP64 value (0 for zero).
 __device__ __forceinline__ int exp_field(double x) {
     return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
@@ -802,57 +776,148 @@ struct Tridiag {
     }
 };
 
+// Each SM quarter issues one FP64 warp instruction per 64 cycles (measured; 32
+// lanes or one), and the scalars between two barriers are one warp's work:
+// powers of two, exponent bounds and FP32 roundings are therefore made on the
+// integer pipe, and what can wait is computed beside the other warps' work.
+__device__ __forceinline__ double pow2i(int e) {
+    return (unsigned)(e + 1022) < 2046u ? __longlong_as_double((long long)(e + 1023) << 52) : ldexp(1.0, e);
+}
+// x 2^de without an FP64 operation where x and the result are normal.
+__device__ __forceinline__ double mul_pow2(double x, int de) {
+    const int e = exp_field(x);
+    if (e > 0 && e < 2047 && (unsigned)(e + de - 1) < 2046u) return __longlong_as_double(__double_as_longlong(x) + ((long long)de << 52));
+    return x == 0.0 ? 0.0 : ldexp(x, de);
+}
+// |c| 2^de, truncated (0 below 2^-100, infinite above 2^100).
+__device__ __forceinline__ float scaled_abs(double c, int de) {
+    const unsigned hi = (unsigned)__double2hiint(c) & 0x7fffffffu, lo = (unsigned)__double2loint(c);
+    const int e = (int)(hi >> 20) + de;
+    if (hi < 0x100000u || e < 923) return 0.0f;
+    if (e > 1123) return INFINITY;
+    return __uint_as_float((unsigned)(e - 896) << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
+}
+// FP64 to FP32, rounded to nearest (ties away), 0 below 2^-126.
+__device__ __forceinline__ float f64_to_f32_near(double x) {
+    return f64_to_f32_trunc(__longlong_as_double(__double_as_longlong(x) + (1ll << 28)));
+}
+// Least exponent field E such that |x| < 2^(E - 1022) for |x| <= r 2^(base - 1022).
+__device__ __forceinline__ int bound_exp(float r, int base) {
+    const unsigned b = __float_as_uint(r);
+    return base + (int)(b >> 23) - 126 - ((b & 0x7fffffu) == 0u ? 1 : 0);
+}
+// 1 / sqrt(x) for normal x > 0: a 23-bit start and one step of third order.
+__device__ __forceinline__ double rsqrt3(double x) {
+    // x = m 2^(2 q), m in [1, 4)
+    const int e = exp_field(x) - 1023, q = e >> 1;
+    const double m = __longlong_as_double(__double_as_longlong(x) - ((long long)(2 * q) << 52));
+    const double y = f32_to_f64_int(rsqrtf(f64_to_f32_trunc(m)));
+    const double r = fma(-m * y, y, 1.0);
+    return mul_pow2(fma(y * r, fma(r, 0.375, 0.5), y), -q);
+}
+__device__ __forceinline__ int bound_exp(double r, int base) {
+    int ex;
+    const double fr = frexp(r, &ex);
+    return base + (fr == 0.5 ? ex - 1 : ex);
+}
+
 // Sum of n partials and the largest of their exponents, in a fixed order, for
-// every thread of the block (every block of a launch gets the same bits).
-// sm: kThreads / 32 entries.
-__device__ __forceinline__ Partial sum_partials(const Partial* p, int n, Partial* sm) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = min((int)blockDim.x, kThreads) >> 5;
-    const int used = min(nw, (n + 31) >> 5);  // warps with anything to add
+// the first warp (every block of a launch gets the same bits).  All threads of
+// the block call it.  The first kThreads threads add n / kThreads partials
+// each, the first warp their sums: 13 FP64 instructions after the first adds,
+// against 5 per warp for a butterfly in every warp.
+struct SumShared {
+    double v[kThreads];
+    int e[kThreads / 32];
+};
+
+__device__ __forceinline__ Partial sum_partials(const Partial* p, int n, SumShared& sm) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double s = 0.0;
     int e = 0;
-    if (warp < used) {
-        for (int i = threadIdx.x; i < n; i += 32 * nw) {
+    if (tid < kThreads) {
+        for (int i = tid; i < n; i += kThreads) {
             const Partial q = p[i];
-            s += q.v;
+            s = i == tid ? q.v : s + q.v;
             e = max(e, (int)q.e);
         }
-        s = warp_sum(s);
-        e = __reduce_max_sync(0xffffffffu, e);
-        if (lane == 0) {
-            sm[warp].v = s;
-            sm[warp].e = e;
+        sm.v[tid] = s;
+        if (32 * warp < n) {
+            e = __reduce_max_sync(0xffffffffu, e);
+            if (lane == 0) sm.e[warp] = e;
         }
     }
     __syncthreads();
-    if (used > 1) {
-        if (warp == 0) {
-            s = lane < used ? sm[lane].v : 0.0;
-            e = lane < used ? (int)sm[lane].e : 0;
-#pragma unroll
-            for (int o = kThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            e = __reduce_max_sync(0xffffffffu, e);
-            __syncwarp();
-            if (lane == 0) {
-                sm[0].v = s;
-                sm[0].e = e;
-            }
-        }
-        __syncthreads();
+    Partial r;
+    r.v = 0.0;
+    r.e = 0;
+    if (warp == 0) {
+        const int used = min(kThreads / 32, (n + 31) / 32);
+        s = sm.v[lane];
+        for (int w = 1; w < used; ++w) s += sm.v[32 * w + lane];
+        r.v = warp_sum(s);
+        e = 0;
+        for (int w = 0; w < used; ++w) e = max(e, sm.e[w]);
+        r.e = e;
     }
-    Partial r = sm[0];
     return r;
 }
 
+// One block's partial sum and largest exponent, stored in *out, in the same
+// manner (kThreads threads; sm may hold the head's sums, which a barrier ended).
+__device__ __forceinline__ void block_partial(double v, int e, SumShared& sm, Partial* out) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    sm.v[tid] = v;
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) sm.e[warp] = e;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) v += sm.v[32 * w + lane];
+        v = warp_sum(v);
+        e = lane < kThreads / 32 ? sm.e[lane] : 0;
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) {
+            out->v = v;
+            out->e = e;
+        }
+    }
+}
+
+// What the head of a kernel computes once per block: the scalars that follow
+// from the previous kernel's partial sums, by the first warp.  An FP64
+// instruction holds its SM quarter's pipe for 64 cycles in every warp that
+// repeats it, so a square root and a division in all warps of all resident
+// blocks delay a short launch by more than its loads.  Ground state and propagation of a
+// 63,504-state star 89.9 -> 76.1 ms, 96 star columns 182 -> 169, gradient of
+// the star 194 -> 172, the 853,776-state ring 14.08 -> 13.74 (its streams hide
+// most of it).
+struct HeadShared {
+    SumShared sum;
+    double aj;         // resolve_alpha: a_j s_j (and araw = a_j)
+    double araw;
+    double scale, cprev;  // resolve_norm: s_j, b_j s_{j-1}
+    int ew, emax, m_eff;
+};
+
 // a_j = <v_j, w> and the largest exponent of w from the partial sums that
 // H*psi left (every block computes the same; `writer` also stores them).
-__device__ __forceinline__ double resolve_alpha(const ColDesc& D, ColScalars* C, bool writer, Partial* sm, int& ew) {
-    const Partial t = sum_partials(D.part_a, C->n_alpha, sm);
-    ew = (int)t.e;
-    if (writer) {
-        C->araw = t.v;
-        C->ew = ew;
+// Ends with a barrier: all threads may read the shared values.
+__device__ __forceinline__ void resolve_alpha(const ColDesc& D, ColScalars* C, int j, bool writer, HeadShared& sh) {
+    const Partial t = sum_partials(D.part_a, C->n_alpha, sh.sum);
+    if (threadIdx.x < 32) {
+        const double aj = t.v * C->scale[j];
+        if (threadIdx.x == 0) {
+            sh.araw = t.v;
+            sh.aj = aj;
+            sh.ew = (int)t.e;
+            if (writer) {
+                C->araw = t.v;
+                C->ew = (int)t.e;
+            }
+        }
     }
-    return t.v;
+    __syncthreads();
 }
 
 // What the update that made V_j (j >= 1) leaves to the next kernel: b_j =
@@ -860,34 +925,42 @@ __device__ __forceinline__ double resolve_alpha(const ColDesc& D, ColScalars* C,
 // test (the Krylov space is invariant when b_j is at rounding level relative
 // to |a_{j-1}| + b_{j-1}).  Every block computes the same values from the
 // partial sums; only `writer` stores them, so no block reads what another
-// may be writing (m_eff takes the same value before and after).
-struct NormHead {
-    double beta, scale;
-    int emax, m_eff;
-};
-
-__device__ __forceinline__ NormHead resolve_norm(const ColDesc& D, ColScalars* C, int j, bool writer, Partial* sm) {
-    NormHead h;
-    h.m_eff = C->m_eff;
-    h.beta = h.scale = 0.0;
-    h.emax = 0;
-    if (j - 1 >= h.m_eff) return h;  // the update did not run (block-uniform)
-    const double a = C->abase + C->hre, ref = fabs(a) + C->beta[j - 1];
-    const Partial t = sum_partials(D.part_n, C->n_norm, sm);
-    h.beta = sqrt(t.v);
-    h.scale = h.beta > 0.0 ? 1.0 / h.beta : 0.0;
-    h.emax = (int)t.e;
-    const bool bad = !isfinite(h.beta) || !isfinite(a);
-    if (bad || h.beta <= 1e-12 * fmax(ref, 1e-300)) h.m_eff = j;  // happy breakdown: K_j is invariant
-    if (writer) {
-        C->alpha[j - 1] = a;
-        C->beta[j] = h.beta;
-        C->scale[j] = h.scale;
-        C->emax[j] = h.emax;
-        C->m_eff = h.m_eff;
-        if (bad) C->status = KG_ENUMERIC;
+// may be writing (m_eff takes the same value before and after).  Ends with a
+// barrier, like resolve_alpha.
+__device__ __forceinline__ void resolve_norm(const ColDesc& D, ColScalars* C, int j, bool writer, HeadShared& sh) {
+    const int m_old = C->m_eff;
+    if (j - 1 >= m_old) {  // the update did not run (block-uniform)
+        if (threadIdx.x == 0) sh.m_eff = m_old;
+        __syncthreads();
+        return;
     }
-    return h;
+    const Partial t = sum_partials(D.part_n, C->n_norm, sh.sum);
+    if (threadIdx.x < 32) {
+        const double a = C->abase + C->hre, ref = 1e-12 * fmax(fabs(a) + C->beta[j - 1], 1e-300);
+        // b_j and 1/b_j from one reciprocal square root, b_j with its last rounding mended
+        const bool some = t.v > 0.0 && exp_field(t.v) != 2047;
+        const double rs = some ? (exp_field(t.v) > 0 ? rsqrt3(t.v) : 1.0 / sqrt(t.v)) : 0.0;
+        const double q = t.v * rs;
+        const double b = some ? fma(0.5 * rs, fma(-q, q, t.v), q) : t.v;  // 0, infinity or NaN
+        const bool bad = exp_field(t.v) == 2047 || exp_field(a) == 2047 || (int)t.e == 2047;
+        const int m = bad || !(b > ref) ? j : m_old;  // happy breakdown: K_j is invariant
+        const double cp = b * C->scale[j - 1];
+        if (threadIdx.x == 0) {
+            sh.scale = rs;
+            sh.cprev = cp;
+            sh.emax = (int)t.e;
+            sh.m_eff = m;
+            if (writer) {
+                C->alpha[j - 1] = a;
+                C->beta[j] = b;
+                C->scale[j] = rs;
+                C->emax[j] = (int)t.e;
+                C->m_eff = m;
+                if (bad) C->status = KG_ENUMERIC;
+            }
+        }
+    }
+    __syncthreads();
 }
 
 // Deterministic reduction over the nblk blocks of one column (block `row`).

@@ -349,18 +349,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_reorth_dots(const ColDesc* desc
     constexpr int TG = kThreads / G;           // threads per group
     __shared__ double sm[(kThreads / 32) * 3 * KH];
     __shared__ double bs[3 * NK], red[3 * NK];
-    __shared__ Partial pair[kThreads / 32];
+    __shared__ HeadShared head;
     KG_ITEM();
     if (j >= C->m_eff) return;
-    int ew;
-    const double araw = second ? 0.0 : resolve_alpha(D, C, blk == 0 && threadIdx.x == 0, pair, ew);
+    if (!second) resolve_alpha(D, C, j, blk == 0 && threadIdx.x == 0, head);
     const int d = D.d;
     const int grp = threadIdx.x / TG, t = threadIdx.x % TG;
     const int kb = grp * KH, kn = min(KH, NK - kb);
     const double2* Vb = D.V + (size_t)(k0 + kb) * d;
     const double2* w = second ? D.V + (size_t)(j + 1) * d : D.W;
     const double2* vj = D.V + (size_t)j * d;
-    const double aj = second ? 0.0 : araw * C->scale[j];
+    const double aj = second ? 0.0 : head.aj;
     double acc[3 * KH];
 #pragma unroll
     for (int k = 0; k < 3 * KH; ++k) acc[k] = 0.0;
@@ -524,7 +523,7 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
     constexpr int KH = P::KH, TG = P::TG, T = P::T, S = P::S;
     extern __shared__ __align__(128) unsigned char dyn[];
     __shared__ __align__(8) unsigned long long full[S], empty[S];
-    __shared__ Partial pair[kThreads / 32];
+    __shared__ HeadShared head;
     __shared__ int eu_s, any_s, fresh_s[NK], ek_s[NK];
     int4* const ua = reinterpret_cast<int4*>(dyn + S * P::kStage);  // [2][kThreads] image of u
     int2* const ub = reinterpret_cast<int2*>(dyn + S * P::kStage + 2 * kThreads * 16);
@@ -571,9 +570,8 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
     };
     if (nr > 0) load_u(0);
     const bool writer = blk == 0 && threadIdx.x == 0;
-    int ew;
-    const double araw = resolve_alpha(D, C, writer, pair, ew);
-    const double aj = araw * C->scale[j];
+    resolve_alpha(D, C, j, writer, head);
+    const double aj = head.aj;
     // the last chunk leaves u = W - a_j v_j in U (which may be W itself)
     const bool keep = k0 + NK == j + 1;
     if (threadIdx.x < NK) {
@@ -588,10 +586,9 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
     }
     if (threadIdx.x == 0) {
         // |u_i| <= |W_i| + |a_j| |V_j[i]| < (1 + |a_j| 2^(E_j - E_w)) 2^(E_w - 1022), with a margin
-        const double r = (1.0 + fabs(aj) * ldexp(1.0, C->emax[j] - ew)) * (1.0 + 1.0 / 1024.0);
-        int ex;
-        const double fr = frexp(r, &ex);
-        eu_s = ew + (fr == 0.5 ? ex - 1 : ex);
+        const int ew = head.ew, ej = C->emax[j];
+        const float r = (1.0f + scaled_abs(aj, ej - ew)) * (1.0f + 1.0f / 1024.0f);
+        eu_s = r < 0x1p120f ? bound_exp(r, ew) : bound_exp((1.0 + fabs(aj) * ldexp(1.0, ej - ew)) * (1.0 + 1.0 / 1024.0), ew);
         if (writer) C->eu = eu_s;
     }
     __syncthreads();
@@ -769,7 +766,7 @@ int launch_reorth_dots(Krylov& K, int j, int k0, int nk, bool second, cudaStream
 __device__ __forceinline__ double2 exact_dot(const ColDesc& D, ColScalars* C, int j, int k, bool keep) {
     const ulonglong2* t = reinterpret_cast<const ulonglong2*>(D.gacc + (size_t)(j & 1) * 4 * (D.M + 1) + 4 * (size_t)k);
     const int em = C->emax[k], ei = C->eimg[k], Ek = ei - em > kFixSlack ? em : ei;
-    const double f = C->scale[k] * ldexp(1.0, Ek + C->eu - 2122);
+    const double f = mul_pow2(C->scale[k], Ek + C->eu - 2122);
     auto val = [](ulonglong2 l) {
         const long long hi = (long long)l.y + (long long)(l.x >> 46);
         return fma((double)hi, 0x1p46, (double)(l.x & ((1ull << 46) - 1ull)));
@@ -791,9 +788,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     __shared__ int idx32[kMaxMgs + 1], idx64[kMaxMgs + 1];
     __shared__ int n32, n64, efix_s;
     __shared__ double hre_s;
-    __shared__ double sm[kThreads / 32];
-    __shared__ int smi[kThreads / 32];
-    __shared__ Partial pair[kThreads / 32];
+    __shared__ HeadShared head;
     KG_ITEM();
     chain_wait();
     if (j >= C->m_eff) return;
@@ -804,37 +799,44 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
     // a_j before the Gram-Schmidt correction: from the dots before a first
     // pass, else (no Gram-Schmidt) straight from the partial sums of H*psi
     int ew = 0;
-    double araw = 0.0;
+    double araw = 0.0, aj = 0.0;
     if (second) {
         ew = C->emax[j + 1];
     } else if (nk) {
         araw = C->araw;
         ew = C->ew;
+        if (threadIdx.x < 32) aj = araw * C->scale[j];  // the first warp's only (below)
     } else {
-        araw = resolve_alpha(D, C, writer, pair, ew);
+        resolve_alpha(D, C, j, writer, head);
+        araw = head.araw;
+        aj = head.aj;
+        ew = head.ew;
     }
-    const double aj = araw * C->scale[j];
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         int a32 = 0, a64 = 0;
         // bound of the result's components, in units of 2^(ew - 1022) (below)
-        double r = 0.0;
+        float r = 0.0f;
         for (int k0 = 0; k0 < nk; k0 += 32) {
             const int k = k0 + lane;
             double2 h = make_double2(0.0, 0.0), c = h;
+            int es = 0;
             if (k < nk) {
                 const double s = C->scale[k];
+                es = exp_field(s);
                 h = exact ? exact_dot(D, C, j, k, blk == 0) : C->h[k];
                 if (k == j) hre_s = h.x;
                 c = make_double2(s * h.x, s * h.y);
-                r += (fabs(c.x) + fabs(c.y)) * ldexp(1.0, C->emax[k] - ew);
+                const int de = C->emax[k] - ew;
+                r += scaled_abs(c.x, de) + scaled_abs(c.y, de);
             }
-            const bool small = (fabs(h.x) + fabs(h.y)) < kSmallCoef;  // |h_k| for the unit vector v_k
+            // |h_k| for the unit vector v_k; a start vector of extreme norm (c or its FP32 copy out of range) stays in FP64
+            const bool small = scaled_abs(h.x, 0) + scaled_abs(h.y, 0) < (float)kSmallCoef && (unsigned)(es - 963) <= 120u;
             const unsigned in = __ballot_sync(0xffffffffu, k < nk), ms = __ballot_sync(0xffffffffu, k < nk && small);
             const unsigned before = (1u << lane) - 1u;
             if (k < nk && small) {
                 const int q = a32 + __popc(ms & before);
-                coef32[q] = make_float2((float)c.x, (float)c.y);
+                coef32[q] = make_float2(f64_to_f32_near(c.x), f64_to_f32_near(c.y));
                 idx32[q] = k;
             } else if (k < nk) {
                 const int q = a64 + __popc(in & ~ms & before);
@@ -844,7 +846,9 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
             a32 += __popc(ms);
             a64 += __popc(in & ~ms);
         }
-        r = warp_sum(r);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        __syncwarp();
         if (lane == 0) {
             n32 = a32;
             n64 = a64;
@@ -852,12 +856,20 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
             //   2^(E_u - 1022) + |a_j| 2^(E_j - 1022) + sum_k (|Re c_k| + |Im c_k|) 2^(E_k - 1022)
             // (E_u: largest exponent of W, or of V_{j+1} in a second pass),
             // times a margin for the rounding of the FP64 and FP32 arithmetic.
-            r += 1.0;
-            if (!second) r += fabs(aj) * ldexp(1.0, C->emax[j] - ew);
-            r *= 1.0 + 1.0 / 1024.0;
-            int ex;
-            const double fr = frexp(r, &ex);  // r = fr * 2^ex, fr in [0.5, 1)
-            efix_s = ew + (fr == 0.5 ? ex - 1 : ex);
+            r += 1.0f;
+            if (!second) r += scaled_abs(aj, C->emax[j] - ew);
+            r *= 1.0f + 1.0f / 1024.0f;
+            if (r < 0x1p120f) {
+                efix_s = bound_exp(r, ew);
+            } else {  // coefficients out of FP32's range
+                double rd = 1.0;
+                if (!second) rd += fabs(aj) * ldexp(1.0, C->emax[j] - ew);
+                for (int q = 0; q < a64; ++q)
+                    rd += (fabs(coef64[q].x) + fabs(coef64[q].y)) * ldexp(1.0, C->emax[idx64[q]] - ew);
+                for (int q = 0; q < a32; ++q)
+                    rd += ((double)fabsf(coef32[q].x) + (double)fabsf(coef32[q].y)) * ldexp(1.0, C->emax[idx32[q]] - ew);
+                efix_s = bound_exp(rd * (1.0 + 1.0 / 1024.0), ew);
+            }
         }
     }
     __syncthreads();
@@ -968,7 +980,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
         KG_FOR(i) element(i);
     }
     chain_next();
-    block_partial(acc, em, sm, smi, D.part_n + blk);
+    block_partial(acc, em, head.sum, D.part_n + blk);
     if (writer) {
         C->n_norm = nblk;
         C->abase = second ? C->alpha[j] : araw;
@@ -981,10 +993,10 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
 
 // resolve_norm by itself, one block per column.
 __global__ void __launch_bounds__(kThreads) k_resolve(const ColDesc* desc, ColScalars* cs, int j) {
-    __shared__ Partial pair[kThreads / 32];
+    __shared__ HeadShared head;
     const ColDesc D = desc[blockIdx.x];
     chain_wait();
-    resolve_norm(D, cs + blockIdx.x, j, threadIdx.x == 0, pair);
+    resolve_norm(D, cs + blockIdx.x, j, threadIdx.x == 0, head);
 }
 
 int launch_resolve(Krylov& K, int j, cudaStream_t st) {
@@ -1457,11 +1469,13 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
 #pragma unroll
         for (int o_ = 16; o_ > 0; o_ >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o_));
         int a64 = 0, a32 = 0;
+        // norms within 2^-60 .. 2^60: the FP32 copies and coefficients neither overflow nor vanish
+        const bool in32 = V32 && (unsigned)(exp_field(cmax) - 963) <= 120u;
         for (int k0 = 0; k0 < m; k0 += 32) {
             const int k = k0 + lane;
             const double2 c = k < m ? C->c[k] : make_double2(0.0, 0.0);
             const double sk = k < m ? C->scale[k] : 0.0;
-            const bool small = V32 && sk > 0.0 && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
+            const bool small = in32 && (unsigned)(exp_field(sk) - 963) <= 120u && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
             const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, k < m && small);
             const unsigned before = (1u << lane) - 1u;
             if (k < m && small) {

@@ -194,51 +194,6 @@ __device__ __forceinline__ void sum_slots(const ulonglong2* slot, int n, unsigne
     l1 = (unsigned long long)b0 + ((unsigned long long)b1 << 27) + ((unsigned long long)b2 << 54);
 }
 
-// Each SM quarter issues one FP64 warp instruction per 64 cycles (measured; 32
-// lanes or one), and the scalars between two barriers are one warp's work:
-// powers of two, exponent bounds and FP32 roundings are therefore made on the
-// integer pipe, and what can wait is computed beside the other warps' work.
-__device__ __forceinline__ double pow2i(int e) {
-    return (unsigned)(e + 1022) < 2046u ? __longlong_as_double((long long)(e + 1023) << 52) : ldexp(1.0, e);
-}
-// x 2^de without an FP64 operation where x and the result are normal.
-__device__ __forceinline__ double mul_pow2(double x, int de) {
-    const int e = exp_field(x);
-    if (e > 0 && e < 2047 && (unsigned)(e + de - 1) < 2046u) return __longlong_as_double(__double_as_longlong(x) + ((long long)de << 52));
-    return x == 0.0 ? 0.0 : ldexp(x, de);
-}
-// |c| 2^de, truncated (0 below 2^-100, infinite above 2^100).
-__device__ __forceinline__ float scaled_abs(double c, int de) {
-    const unsigned hi = (unsigned)__double2hiint(c) & 0x7fffffffu, lo = (unsigned)__double2loint(c);
-    const int e = (int)(hi >> 20) + de;
-    if (hi < 0x100000u || e < 923) return 0.0f;
-    if (e > 1123) return INFINITY;
-    return __uint_as_float((unsigned)(e - 896) << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
-}
-// FP64 to FP32, rounded to nearest (ties away), 0 below 2^-126.
-__device__ __forceinline__ float f64_to_f32_near(double x) {
-    return f64_to_f32_trunc(__longlong_as_double(__double_as_longlong(x) + (1ll << 28)));
-}
-// Least exponent field E such that |x| < 2^(E - 1022) for |x| <= r 2^(base - 1022).
-__device__ __forceinline__ int bound_exp(float r, int base) {
-    const unsigned b = __float_as_uint(r);
-    return base + (int)(b >> 23) - 126 - ((b & 0x7fffffu) == 0u ? 1 : 0);
-}
-// 1 / sqrt(x) for normal x > 0: a 23-bit start and one step of third order.
-__device__ __forceinline__ double rsqrt3(double x) {
-    // x = m 2^(2 q), m in [1, 4)
-    const int e = exp_field(x) - 1023, q = e >> 1;
-    const double m = __longlong_as_double(__double_as_longlong(x) - ((long long)(2 * q) << 52));
-    const double y = f32_to_f64_int(rsqrtf(f64_to_f32_trunc(m)));
-    const double r = fma(-m * y, y, 1.0);
-    return mul_pow2(fma(y * r, fma(r, 0.375, 0.5), y), -q);
-}
-__device__ __forceinline__ int bound_exp(double r, int base) {
-    int ex;
-    const double fr = frexp(r, &ex);
-    return base + (fr == 0.5 ? ex - 1 : ex);
-}
-
 // What the scalar warp tells the block.
 struct SmallShared {
     SecView S;

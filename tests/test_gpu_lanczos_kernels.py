@@ -74,6 +74,18 @@ def test_small_columns_equal_streaming(name, L, nu, nd, M):
         assert np.max(np.abs(y - oracle.Sector(m).propagate(x, 0.12))) < TOL
 
 
+@pytest.mark.parametrize("schedule", [2, 4])  # the streaming kernels, exact and FP64 dots
+@pytest.mark.parametrize("p2", [-400, -130, -61, 61, 130, 400])
+def test_scaled_start(p2, schedule):
+    """A start vector scaled by a power of two, far enough to leave FP32's
+    range in its coefficients and copies, gives the scaled result."""
+    m = W.random_model(9, 4, 4, seed=20, complex_hopping=True)
+    x = W.random_state(W.sector_dim(9, 4, 4), 20)
+    y = propagate(m, x, 0.02, 2, M=20, schedule=schedule)
+    z = propagate(m, x * 2.0 ** p2, 0.02, 2, M=20, schedule=schedule)
+    assert np.max(np.abs(z * 2.0 ** -p2 - y)) < TOL
+
+
 def test_small_column_near_breakdown():
     """A start vector that spans three eigenvectors to 1e-9: the space is
     nearly invariant after three vectors, so the images' exponent bounds are
