@@ -35,34 +35,52 @@
 
 namespace kg {
 
-constexpr int kMaxNodes = 16;
+constexpr int kNodes = 10;       // Gauss-Legendre nodes of a step
+constexpr int kGradThreads = 64;  // threads per block of k_param_grad
+constexpr int kGradBlocks = 152 * 16;
 constexpr int kMaxPairs = 128;
 
 // ------------------------------------------------------- node vectors
 // out[outoff[b] + t*d_b + i] = sum_k cq[b][t][k] V_k[i] for every column b
-// of K (columns may differ in dimension d_b).
-__global__ void __launch_bounds__(kThreads) k_lincomb(const ColDesc* desc, const ColScalars* cs, int Mcap,
-                                                      const double2* cq, int ntau, double2* out,
-                                                      const size_t* outoff) {
-    __shared__ double2 c[kMaxNodes + 1][kMaxM];
+// of K (columns may differ in dimension d_b) and t < NT.  Bound by the FP64
+// pipe (4 m NT multiply-adds per element), with the sums in registers.
+template <int NT>
+__global__ void __launch_bounds__(kGradThreads) k_lincomb(const ColDesc* desc, const ColScalars* cs, int Mcap,
+                                                          const double2* cq, double2* out, const size_t* outoff) {
+    __shared__ double2 c[kMaxM][NT];
     const int b = blockIdx.y;
     const ColDesc D = desc[b];
     const int m = cs[b].m_eff;
-    for (int t = 0; t < ntau; ++t)
-        for (int k = threadIdx.x; k < m; k += blockDim.x) c[t][k] = cq[((size_t)b * ntau + t) * Mcap + k];
+    for (int q = threadIdx.x; q < NT * m; q += blockDim.x) c[q % m][q / m] = cq[((size_t)b * NT + q / m) * Mcap + q % m];
     __syncthreads();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < D.d; i += gridDim.x * blockDim.x) {
-        double2 acc[kMaxNodes + 1];
-        for (int t = 0; t < ntau; ++t) acc[t] = make_double2(0.0, 0.0);
+        double2 acc[NT];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) acc[t] = make_double2(0.0, 0.0);
+#pragma unroll 2
         for (int k = 0; k < m; ++k) {
             const double2 v = D.V[(size_t)k * D.d + i];
-            for (int t = 0; t < ntau; ++t) {
-                acc[t].x = fma(c[t][k].x, v.x, fma(-c[t][k].y, v.y, acc[t].x));
-                acc[t].y = fma(c[t][k].x, v.y, fma(c[t][k].y, v.x, acc[t].y));
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const double2 a = c[k][t];
+                acc[t].x = fma(a.x, v.x, fma(-a.y, v.y, acc[t].x));
+                acc[t].y = fma(a.x, v.y, fma(a.y, v.x, acc[t].y));
             }
         }
-        for (int t = 0; t < ntau; ++t) out[outoff[b] + (size_t)t * D.d + i] = acc[t];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) out[outoff[b] + (size_t)t * D.d + i] = acc[t];
     }
+}
+
+template <int NT>
+static int launch_lincomb(const Krylov& K, const double2* cq, double2* out, const size_t* outoff, cudaStream_t st) {
+    int d = 1;
+    for (auto& D : K.hdesc) d = std::max(d, (int)D.d);
+    ProfScope ps("lincomb", st);
+    k_lincomb<NT><<<dim3(std::min(kGradBlocks, (d + kGradThreads - 1) / kGradThreads), K.B), kGradThreads, 0, st>>>(
+        K.desc, K.cs, K.M, cq, out, outoff);
+    KG_LAUNCHED();
+    return KG_OK;
 }
 
 // ---------------------------------------------------- parameter gradient
@@ -72,15 +90,27 @@ __global__ void __launch_bounds__(kThreads) k_lincomb(const ColDesc* desc, const
 //   g[3L + 2p (+1)]     += Re (Im) sum_q c_q <w_q| sum_sigma c^dag_a c_b |u_q>
 // for every ordered hop pair p = (a, b) of the sector's hop tables.
 struct NodeWeights {
-    double2 c[kMaxNodes];
+    double2 c[kNodes];
 };
 
-__global__ void __launch_bounds__(kThreads) k_param_grad(SecView S, const double2* __restrict__ U,
-                                                         const double2* __restrict__ Wv, NodeWeights wts, int nq,
-                                                         const short* __restrict__ pairmap, int nparam,
-                                                         double* partial) {
+//
+// One state per thread as long as the grid lasts.  Bound by the FP64 pipe:
+// 4 NQ multiply-adds per hop.  A butterfly per parameter would add 5 adds per
+// parameter and warp (as many as a third of the products for 66 parameters
+// and 10 nodes), so the warp transposes 32 parameters at a time through
+// shared memory and each lane adds up one of them (a tail of few parameters
+// is split over the lanes).  Blocks of two warps spread 63,504 states evenly.
+// With the blocks' sums added by a warp per parameter, a pass over 63,504
+// states with 10 nodes and 66 parameters went from 200 to 83 us (FP64: 65).
+template <int NQ>
+__global__ void __launch_bounds__(kGradThreads) k_param_grad(SecView S, const double2* __restrict__ U,
+                                                             const double2* __restrict__ Wv, NodeWeights wts,
+                                                             const short* __restrict__ pairmap, int nparam,
+                                                             double* partial) {
+    constexpr int kWarps = kGradThreads / 32;
     __shared__ short pm[kMaxL * kMaxL];
-    __shared__ double sm[(kThreads / 32) * (3 * kMaxL + 2 * kMaxPairs)];
+    __shared__ double tile[kWarps][32 * 33];
+    __shared__ double sm[kWarps * (3 * kMaxL + 2 * kMaxPairs)];
     for (int k = threadIdx.x; k < S.L * S.L; k += blockDim.x) pm[k] = pairmap[k];
     __syncthreads();
     const int L = S.L;
@@ -89,9 +119,10 @@ __global__ void __launch_bounds__(kThreads) k_param_grad(SecView S, const double
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.d; s += gridDim.x * blockDim.x) {
         int i_dn, i_up;
         split_index(S, s, i_dn, i_up);
-        double2 a[kMaxNodes];  // c_q conj(w_q[s])
+        double2 a[NQ];  // c_q conj(w_q[s])
         double P = 0.0;
-        for (int q = 0; q < nq; ++q) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
             const double2 w = Wv[(size_t)q * S.d + s], u = U[(size_t)q * S.d + s];
             const double2 c = wts.c[q];
             a[q] = make_double2(c.x * w.x + c.y * w.y, c.y * w.x - c.x * w.y);
@@ -108,10 +139,11 @@ __global__ void __launch_bounds__(kThreads) k_param_grad(SecView S, const double
                 const uint2 en = pass == 0 ? S.up_ent[e] : S.dn_ent[e];
                 const size_t src = pass == 0 ? (size_t)i_dn * S.Du + en.x : (size_t)en.x * S.Du + i_up;
                 double zr = 0.0, zi = 0.0;
-                for (int q = 0; q < nq; ++q) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
                     const double2 u = U[(size_t)q * S.d + src];
-                    zr += a[q].x * u.x - a[q].y * u.y;
-                    zi += a[q].x * u.y + a[q].y * u.x;
+                    zr = fma(a[q].x, u.x, fma(-a[q].y, u.y, zr));
+                    zi = fma(a[q].x, u.y, fma(a[q].y, u.x, zi));
                 }
                 if (en.y >> 31) {
                     zr = -zr;
@@ -123,26 +155,41 @@ __global__ void __launch_bounds__(kThreads) k_param_grad(SecView S, const double
             }
         }
     }
-    // block reduction in a fixed order: warp sums, then warps in order
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int p = 0; p < nparam; ++p) {
-        const double v = warp_sum(acc[p]);
-        if (lane == 0) sm[warp * nparam + p] = v;
+    // block reduction in a fixed order
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* const t = tile[warp];
+    for (int p0 = 0; p0 < nparam; p0 += 32) {
+        const int n = min(32, nparam - p0);
+        for (int r = 0; r < n; ++r) t[33 * r + lane] = acc[p0 + r];
+        __syncwarp();
+        int w = 1;  // lanes with one part each of w >= n parameters
+        while (w < n) w *= 2;
+        const int r = lane & (w - 1), g = lane / w;
+        double v = 0.0;
+        if (r < n) {
+            v = t[33 * r + g * w];
+            for (int i = 1; i < w; ++i) v += t[33 * r + g * w + i];
+        }
+        for (int o = w; o < 32; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane < n) sm[warp * nparam + p0 + lane] = v;
+        __syncwarp();
     }
     __syncthreads();
     for (int p = threadIdx.x; p < nparam; p += blockDim.x) {
-        double t = 0.0;
-        for (int w = 0; w < nw; ++w) t += sm[w * nparam + p];
-        partial[(size_t)blockIdx.x * nparam + p] = t;
+        double v = sm[p];
+        for (int w = 1; w < kWarps; ++w) v += sm[w * nparam + p];
+        partial[(size_t)p * gridDim.x + blockIdx.x] = v;
     }
 }
 
+// g[p] += the sum of the blocks' partials, one warp per parameter.
 __global__ void k_param_reduce(const double* partial, int nblk, int nparam, double* g) {
-    for (int p = threadIdx.x; p < nparam; p += blockDim.x) {
-        double t = 0.0;
-        for (int b = 0; b < nblk; ++b) t += partial[(size_t)b * nparam + p];
-        g[p] += t;
-    }
+    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (p >= nparam) return;
+    double t = 0.0;
+    for (int b = lane; b < nblk; b += 32) t += partial[(size_t)p * nblk + b];
+    t = warp_sum(t);
+    if (lane == 0) g[p] += t;
 }
 
 // ----------------------------------------------------------- utilities
@@ -290,14 +337,18 @@ static ParamMap param_map(const kg_sector* s) {
 }
 
 static int grad_pass(const kg_sector* sec, const double2* U, const double2* Wv, const std::vector<std::complex<double>>& c,
-                     const short* dmap, const ParamMap& P, double* partial, int nblk, double* g, cudaStream_t st) {
+                     const short* dmap, const ParamMap& P, double* partial, double* g, cudaStream_t st) {
     NodeWeights wts;
-    const int nq = (int)c.size();
+    const int nq = (int)c.size();  // kNodes, or 1 for a single pair
     for (int q = 0; q < nq; ++q) wts.c[q] = make_double2(c[q].real(), c[q].imag());
+    const int nblk = (int)std::min<long long>(kGradBlocks, ((long long)sec->d + kGradThreads - 1) / kGradThreads);
     ProfScope ps("param_grad", st);
-    k_param_grad<<<nblk, kThreads, 0, st>>>(sec->view(), U, Wv, wts, nq, dmap, P.nparam, partial);
+    if (nq == kNodes)
+        k_param_grad<kNodes><<<nblk, kGradThreads, 0, st>>>(sec->view(), U, Wv, wts, dmap, P.nparam, partial);
+    else
+        k_param_grad<1><<<nblk, kGradThreads, 0, st>>>(sec->view(), U, Wv, wts, dmap, P.nparam, partial);
     KG_LAUNCHED();
-    k_param_reduce<<<1, 256, 0, st>>>(partial, nblk, P.nparam, g);
+    k_param_reduce<<<(P.nparam + 7) / 8, 256, 0, st>>>(partial, nblk, P.nparam, g);
     KG_LAUNCHED();
     return KG_OK;
 }
@@ -318,7 +369,7 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
     if (!s->has_gs) KG_TRY(ground_state(s, o));
     const int Kc = std::max(1, checkpoint > 0 ? checkpoint : 20);
     cudaStream_t st = pick_stream(s, o);
-    const int L = s->L, d0 = (int)s->d, rows = n_steps + 1, nq = 10;
+    const int L = s->L, d0 = (int)s->d, rows = n_steps + 1, nq = kNodes;
     const ParamMap P = param_map(s);
     if (P.npairs > kMaxPairs) {
         set_error("too many hopping pairs for the adjoint (%d > %d)", P.npairs, kMaxPairs);
@@ -327,12 +378,11 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
     std::vector<double> xq, wq;
     gauss_legendre(nq, xq, wq);
     const double E0 = s->E0;
-    const int nblk = 152 * 2;
     double *g = nullptr, *partial = nullptr;
     short* dmap = nullptr;
     double2* z = nullptr;
     KG_CUDA(cudaMalloc(&g, sizeof(double) * P.nparam));
-    KG_CUDA(cudaMalloc(&partial, sizeof(double) * P.nparam * nblk));
+    KG_CUDA(cudaMalloc(&partial, sizeof(double) * P.nparam * kGradBlocks));
     KG_CUDA(cudaMalloc(&dmap, sizeof(short) * kMaxL * kMaxL));
     KG_CUDA(cudaMalloc(&z, sizeof(double2) * d0));
     KG_CUDA(cudaMemsetAsync(g, 0, sizeof(double) * P.nparam, st));
@@ -644,22 +694,14 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
                     if (rc == KG_OK) rc = build_space(KF, o->reorth, st);
                 }
                 if (rc == KG_OK) rc = launch_tridiag_multi(KF, tauF, nq, cqF, st);
-                if (rc == KG_OK) {
-                    k_lincomb<<<dim3(grid_for((int)(tot / NC) + 1), NC), kThreads, 0, st>>>(KF.desc, KF.cs, KF.M, cqF,
-                                                                                         nq, Uq, offU);
-                    KG_LAUNCHED();
-                }
+                if (rc == KG_OK) rc = launch_lincomb<kNodes>(KF, cqF, Uq, offU, st);
                 // backward space of lambda_k: node vectors w_q and U^dag lambda_k
                 if (rc == KG_OK) rc = load(KB, lam);
                 if (rc == KG_OK) rc = build_space(KB, o->reorth, st);
                 if (rc == KG_OK) rc = launch_tridiag_multi(KB, tauB, nq + 1, cqB, st);
-                if (rc == KG_OK) {
-                    k_lincomb<<<dim3(grid_for((int)(tot / NC) + 1), NC), kThreads, 0, st>>>(KB.desc, KB.cs, KB.M, cqB,
-                                                                                         nq + 1, Wq, offW);
-                    KG_LAUNCHED();
-                }
+                if (rc == KG_OK) rc = launch_lincomb<kNodes + 1>(KB, cqB, Wq, offW, st);
                 for (int b = 0; rc == KG_OK && b < NC; ++b)
-                    rc = grad_pass(grp[colg[b]].nb, Uq + hOffU[b], Wq + hOffW[b], cw[colg[b]], dmap, P, partial, nblk,
+                    rc = grad_pass(grp[colg[b]].nb, Uq + hOffU[b], Wq + hOffW[b], cw[colg[b]], dmap, P, partial,
                                    g, st);
                 // lambda_{k-1} = U^dag lambda_k + s_{k-1}
                 for (int b = 0; rc == KG_OK && b < NC; ++b)
@@ -699,9 +741,9 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
     double2* x = nullptr;
     if (rc == KG_OK && cudaMalloc(&x, sizeof(double2) * d0) != cudaSuccess) rc = KG_ENOMEM;
     if (x) frees.push_back(x);
-    if (rc == KG_OK) rc = grad_pass(s, s->gs, s->gs, {std::complex<double>(Ebar, 0.0)}, dmap, P, partial, nblk, g, st);
+    if (rc == KG_OK) rc = grad_pass(s, s->gs, s->gs, {std::complex<double>(Ebar, 0.0)}, dmap, P, partial, g, st);
     if (rc == KG_OK) rc = cg_projected(s, s->gs, s->E0, z, x, 1e-13, 20000, st);
-    if (rc == KG_OK) rc = grad_pass(s, s->gs, x, {std::complex<double>(-1.0, 0.0)}, dmap, P, partial, nblk, g, st);
+    if (rc == KG_OK) rc = grad_pass(s, s->gs, x, {std::complex<double>(-1.0, 0.0)}, dmap, P, partial, g, st);
     std::vector<double> hg(P.nparam);
     if (rc == KG_OK)
         rc = cudaMemcpyAsync(hg.data(), g, sizeof(double) * P.nparam, cudaMemcpyDeviceToHost, st) == cudaSuccess &&

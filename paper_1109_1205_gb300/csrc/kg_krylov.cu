@@ -1332,86 +1332,52 @@ __global__ void __launch_bounds__(kLowThreads) k_lowest(ColScalars* cs, int Mcap
 
 // ------------------------------------ step exponential by a Taylor series
 // c = beta0 e^{-i T tau} e_1 (times s_k per component) by Tridiag::advance, one
-// warp per column.  Modes 0 and 2 as in k_tridiag.
-constexpr int kMaxTaus = 32;  // times per column in one mode-2 launch
-
+// warp per column, and per time in mode 2.  Modes 0 and 2 as in
+// k_tridiag.  A warp is a serial chain of FP64 instructions: taking the 10
+// or 11 quadrature times of a column in order, each from the one before, took
+// about 100 us a launch; side by side, all from e_1, it is about 15.
 template <int R>
 __global__ void __launch_bounds__(32 * kTriWarps) k_texp(const ColDesc* desc, ColScalars* cs, int B, int Mcap,
                                                         int mode, const double* taus, int ntau, double2* cq) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * kTriWarps + warp;
+    const int item = blockIdx.x * kTriWarps + warp, t = item / B, b = item % B;
     chain_wait();
-    if (b >= B) return;
+    if (t >= ntau) return;
     ColScalars* C = cs + b;
     const int m = C->m_eff;
-    if (m == 0) {
-        for (int k = lane; k < Mcap; k += 32) C->c[k] = make_double2(0.0, 0.0);
-        if (mode == 2)
-            for (int t = 0; t < ntau; ++t)
-                for (int k = lane; k < Mcap; k += 32) cq[((size_t)b * ntau + t) * Mcap + k] = make_double2(0.0, 0.0);
-        return;
-    }
-    Tridiag<R> T;
-    T.load(C->alpha, C->beta, m, lane);
-    const double beta0 = C->beta0;
-    const int nt = mode == 0 ? 1 : ntau;
-    // Several times of one sign (mode 2: quadrature nodes) are taken in order
-    // of |tau|, each from the previous result: e^{-iT t_n} e_1 =
-    // e^{-iT (t_n - t_{n-1})} e^{-iT t_{n-1}} e_1.  Times of mixed signs
-    // restart from e_1.
-    int order[kMaxTaus];
-    for (int t = 0; t < nt; ++t) order[t] = t;
-    if (mode == 2)
-        for (int a1 = 1; a1 < nt; ++a1)  // insertion sort by |tau| (nt <= kMaxTaus)
-            for (int a2 = a1; a2 > 0 && fabs(taus[(size_t)b * ntau + order[a2]]) <
-                                            fabs(taus[(size_t)b * ntau + order[a2 - 1]]); --a2) {
-                const int tmp = order[a2];
-                order[a2] = order[a2 - 1];
-                order[a2 - 1] = tmp;
-            }
+    double2* const out = mode == 0 ? C->c : cq + ((size_t)b * ntau + t) * Mcap;
+    const double tau = mode == 0 ? desc[b].tau : taus[(size_t)b * ntau + t];
     double2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = make_double2((lane + 32 * r) == 0 ? 1.0 : 0.0, 0.0);
-    double tprev = 0.0;
-    for (int tt = 0; tt < nt; ++tt) {
-        const int t = order[tt];
-        const double tfull = mode == 0 ? desc[b].tau : taus[(size_t)b * ntau + t];
-        if (tfull * tprev < 0.0) {  // sign change: start again from e_1
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = make_double2((lane + 32 * r) == 0 ? 1.0 : 0.0, 0.0);
-            tprev = 0.0;
-        }
-        const double tau = tfull - tprev;
-        tprev = tfull;
+    bool ok = m > 0;
+    if (ok) {
+        Tridiag<R> T;
+        T.load(C->alpha, C->beta, m, lane);
         // a non-finite or absurdly large T (more than kMaxSub sub-steps)
         // cannot be exponentiated this way: report it instead of looping
-        if (!T.advance(tau, v, lane, tau == tfull)) {
-            if (lane == 0) C->status = KG_ENUMERIC;
-            for (int k = lane; k < Mcap; k += 32) C->c[k] = make_double2(0.0, 0.0);
-            if (mode == 2)
-                for (int t2 = 0; t2 < ntau; ++t2)
-                    for (int k = lane; k < Mcap; k += 32) cq[((size_t)b * ntau + t2) * Mcap + k] = make_double2(0.0, 0.0);
-            return;
-        }
+        ok = T.advance(tau, v, lane, true);
+        if (!ok && lane == 0) C->status = KG_ENUMERIC;
+    }
+    if (!ok) {
+        for (int k = lane; k < Mcap; k += 32) C->c[k] = out[k] = make_double2(0.0, 0.0);
+        return;
+    }
+    const double beta0 = C->beta0;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = lane + 32 * r;
-            if (k < m) {
-                const double sc = beta0 * C->scale[k];
-                const double2 cv = make_double2(sc * v[r].x, sc * v[r].y);
-                if (mode == 0)
-                    C->c[k] = cv;
-                else
-                    cq[((size_t)b * ntau + t) * Mcap + k] = cv;
-            } else if (k < Mcap && mode == 2) {
-                cq[((size_t)b * ntau + t) * Mcap + k] = make_double2(0.0, 0.0);
-            }
+    for (int r = 0; r < R; ++r) {
+        const int k = lane + 32 * r;
+        if (k < m) {
+            const double sc = beta0 * C->scale[k];
+            out[k] = make_double2(sc * v[r].x, sc * v[r].y);
+        } else if (k < Mcap && mode == 2) {
+            out[k] = make_double2(0.0, 0.0);
         }
     }
 }
 
 static int launch_texp(Krylov& K, int mode, const double* taus, int ntau, double2* cq, cudaStream_t st) {
-    const int nb = (K.B + kTriWarps - 1) / kTriWarps;
+    const int nb = (K.B * ntau + kTriWarps - 1) / kTriWarps;
     return launch_chained(K.M <= 32 ? &k_texp<1> : &k_texp<2>, nb, 32 * kTriWarps, 0, st, K.desc, K.cs, K.B, K.M, mode,
                           taus, ntau, cq);
 }
@@ -1419,7 +1385,7 @@ static int launch_texp(Krylov& K, int mode, const double* taus, int ntau, double
 int launch_tridiag(Krylov& K, int mode, cudaStream_t st) {
     const int nb = (K.B + kTriWarps - 1) / kTriWarps;
     ProfScope ps("tridiag", st);
-    if (mode == 0 && !(K.schedule & 2)) return launch_texp(K, 0, nullptr, 0, nullptr, st);
+    if (mode == 0 && !(K.schedule & 2)) return launch_texp(K, 0, nullptr, 1, nullptr, st);
     if (mode == 1) {
         k_lowest<<<K.B, kLowThreads, 0, st>>>(K.cs, K.M);
         KG_LAUNCHED();
@@ -1618,6 +1584,7 @@ __global__ void __launch_bounds__(kThreads) k_rq(const double2* x, const double2
 
 // Coefficients of exp(-i H t) v_0 for ntau times per column (taus[b][t]),
 // into cq[b][t][0..M) (already times the scales of the stored vectors).
+constexpr int kMaxTaus = 32;  // times per column in one launch
 int launch_tridiag_multi(Krylov& K, const double* taus, int ntau, double2* cq, cudaStream_t st) {
     if (ntau < 1 || ntau > kMaxTaus) {
         set_error("between 1 and %d times per column", kMaxTaus);
