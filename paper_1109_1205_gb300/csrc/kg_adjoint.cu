@@ -43,32 +43,94 @@ constexpr int kMaxPairs = 128;
 // ------------------------------------------------------- node vectors
 // out[outoff[b] + t*d_b + i] = sum_k cq[b][t][k] V_k[i] for every column b
 // of K (columns may differ in dimension d_b) and t < NT.  Bound by the FP64
-// pipe (4 m NT multiply-adds per element), with the sums in registers.
+// pipe, 4 NT multiply-adds per vector and element, with the sums in registers.
+// As in k_combine, a vector whose coefficients on the unit vector v_k are all
+// below 1e-10 of the column's norm is summed in FP32 (an error below 1e-17 of
+// the norm): with 20 vectors a step's exponential has about eight above.
 template <int NT>
 __global__ void __launch_bounds__(kGradThreads) k_lincomb(const ColDesc* desc, const ColScalars* cs, int Mcap,
                                                           const double2* cq, double2* out, const size_t* outoff) {
     __shared__ double2 c[kMaxM][NT];
+    __shared__ float2 c32[kMaxM][NT];
+    __shared__ int idx[kMaxM];  // the FP64 terms' vectors from the front, the FP32 terms' from the back
+    __shared__ int n64_s;
     const int b = blockIdx.y;
     const ColDesc D = desc[b];
-    const int m = cs[b].m_eff;
-    for (int q = threadIdx.x; q < NT * m; q += blockDim.x) c[q % m][q / m] = cq[((size_t)b * NT + q / m) * Mcap + q % m];
+    const ColScalars* C = cs + b;
+    const int m = C->m_eff;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const double beta0 = C->beta0;
+        const int eb = exp_field(beta0);
+        int n64 = 0, n32 = 0;
+        for (int k0 = 0; k0 < m; k0 += 32) {
+            const int k = k0 + lane;
+            const double2* ck = cq + (size_t)b * NT * Mcap + k;
+            bool small = false;
+            if (k < m) {
+                // both norms within 2^-60 .. 2^60: the FP32 copies neither overflow nor vanish
+                const double sk = C->scale[k];
+                const int es = exp_field(sk);
+                float big = 0.0f;
+                for (int t = 0; t < NT; ++t) {
+                    const double2 v = ck[(size_t)t * Mcap];
+                    big = fmaxf(big, scaled_abs(v.x, 0) + scaled_abs(v.y, 0));
+                }
+                small = (unsigned)(es - 963) <= 120u && (unsigned)(eb - 963) <= 120u &&
+                        big < 1e-10f * (scaled_abs(beta0, 0) * scaled_abs(sk, 0));
+            }
+            const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, small);
+            const unsigned before = (1u << lane) - 1u;
+            if (k < m) idx[small ? kMaxM - 1 - n32 - __popc(ms & before) : n64 + __popc(in & ~ms & before)] = k;
+            n64 += __popc(in & ~ms);
+            n32 += __popc(ms);
+        }
+        if (lane == 0) n64_s = n64;
+    }
+    __syncthreads();
+    const int n64 = n64_s, n32 = m - n64;
+    for (int q = threadIdx.x; q < NT * m; q += blockDim.x) {
+        const int r = q / NT, t = q % NT;
+        const double2 v = cq[((size_t)b * NT + t) * Mcap + (r < n64 ? idx[r] : idx[kMaxM - 1 - (r - n64)])];
+        if (r < n64)
+            c[r][t] = v;
+        else
+            c32[r - n64][t] = make_float2(f64_to_f32_near(v.x), f64_to_f32_near(v.y));
+    }
     __syncthreads();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < D.d; i += gridDim.x * blockDim.x) {
         double2 acc[NT];
+        float2 a32[NT];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) acc[t] = make_double2(0.0, 0.0);
+        for (int t = 0; t < NT; ++t) {
+            acc[t] = make_double2(0.0, 0.0);
+            a32[t] = make_float2(0.0f, 0.0f);
+        }
 #pragma unroll 2
-        for (int k = 0; k < m; ++k) {
-            const double2 v = D.V[(size_t)k * D.d + i];
+        for (int r = 0; r < n32; ++r) {
+            const double2 v = D.V[(size_t)idx[kMaxM - 1 - r] * D.d + i];
+            const float vx = f64_to_f32_trunc(v.x), vy = f64_to_f32_trunc(v.y);
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
-                const double2 a = c[k][t];
+                const float2 a = c32[r][t];
+                a32[t].x = fmaf(a.x, vx, fmaf(-a.y, vy, a32[t].x));
+                a32[t].y = fmaf(a.x, vy, fmaf(a.y, vx, a32[t].y));
+            }
+        }
+#pragma unroll 2
+        for (int r = 0; r < n64; ++r) {
+            const double2 v = D.V[(size_t)idx[r] * D.d + i];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const double2 a = c[r][t];
                 acc[t].x = fma(a.x, v.x, fma(-a.y, v.y, acc[t].x));
                 acc[t].y = fma(a.x, v.y, fma(a.y, v.x, acc[t].y));
             }
         }
 #pragma unroll
-        for (int t = 0; t < NT; ++t) out[outoff[b] + (size_t)t * D.d + i] = acc[t];
+        for (int t = 0; t < NT; ++t)
+            out[outoff[b] + (size_t)t * D.d + i] =
+                make_double2(acc[t].x + f32_to_f64_int(a32[t].x), acc[t].y + f32_to_f64_int(a32[t].y));
     }
 }
 
