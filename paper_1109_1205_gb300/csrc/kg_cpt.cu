@@ -497,7 +497,8 @@ int necpt_occupations(kg_sector* ini, kg_sector* fin, int L_b, double T_b, doubl
         set_error("NE-CPT: contour matrices of %d points do not fit", n);
         return done(KG_ENOMEM);
     }
-    if (cudaMemcpy(Wk.M, D.data(), sizeof(double2) * nn, cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(Wk.M, D.data(), sizeof(double2) * nn, cudaMemcpyHostToDevice) != cudaSuccess ||
+        uploads_done() != cudaSuccess)
         return done(cuda_fail(cudaGetLastError(), "NE-CPT bath upload", __FILE__, __LINE__));
     for (int spin = 0; spin < 2; ++spin) {
         const int rc = necpt_spin(ini, fin, spin, C, beta, o, Wk, st, n_out);

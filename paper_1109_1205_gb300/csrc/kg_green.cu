@@ -633,6 +633,7 @@ struct GramPlan {
             return KG_ENOMEM;
         }
         KG_CUDA(cudaMemcpy(tiles, v.data(), sizeof(int2) * ntile, cudaMemcpyHostToDevice));
+        KG_CUDA(uploads_done());
         return KG_OK;
     }
     int run(const double2* X, int d, int nsm, double2* G, cudaStream_t st) const {
@@ -1283,6 +1284,7 @@ static int drive_upload(kg_keldysh* X, const double* dparams, int n_steps) {
     if (ex.empty()) return KG_OK;
     KG_CUDA(cudaMalloc(&X->drive, sizeof(double) * ex.size()));
     KG_CUDA(cudaMemcpy(X->drive, ex.data(), sizeof(double) * ex.size(), cudaMemcpyHostToDevice));
+    KG_CUDA(uploads_done());
     return KG_OK;
 }
 

@@ -390,6 +390,14 @@ const char* last_error();
 
 }  // namespace kg
 
+namespace kg {
+// Waits for the copies and clears that were queued on the legacy stream.  A
+// cudaMemcpy from pageable memory may return once the data is staged, before
+// it has reached the device, and a cudaMemset before it has run; the kernels
+// run on non-blocking streams, which do not wait for either.
+inline cudaError_t uploads_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+}  // namespace kg
+
 // ----------------------------------------------------- device helpers
 #ifdef __CUDACC__
 namespace kg {

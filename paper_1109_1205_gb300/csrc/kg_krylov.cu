@@ -188,6 +188,7 @@ int krylov_alloc(Krylov& K, const std::vector<const kg_sector*>& cols, int M, in
     }
     KG_TRY(need(cudaMemcpy(K.secs, K.hsec.data(), sizeof(SecView) * K.B, cudaMemcpyHostToDevice), "upload"));
     KG_TRY(need(cudaMemcpy(K.desc, K.hdesc.data(), sizeof(ColDesc) * K.B, cudaMemcpyHostToDevice), "upload"));
+    KG_TRY(need(uploads_done(), "upload"));
     return KG_OK;
 }
 
@@ -199,6 +200,7 @@ int krylov_upload(Krylov& K, cudaStream_t st) {
 int krylov_set_diag(Krylov& K, const double* diag) {
     for (auto& S : K.hsec) S.diag = diag;
     KG_CUDA(cudaMemcpy(K.secs, K.hsec.data(), sizeof(SecView) * K.B, cudaMemcpyHostToDevice));
+    KG_CUDA(uploads_done());
     return KG_OK;
 }
 
@@ -265,6 +267,7 @@ int work_list(Krylov& K, const void* kern, int mode, const int4** items, int* n,
         if (!v.empty()) {
             KG_CUDA(cudaMalloc(&d, sizeof(int4) * v.size()));
             KG_CUDA(cudaMemcpy(d, v.data(), sizeof(int4) * v.size(), cudaMemcpyHostToDevice));
+            KG_CUDA(uploads_done());
         }
         it = K.lists.emplace(key, std::make_pair(d, (int)v.size())).first;
     }

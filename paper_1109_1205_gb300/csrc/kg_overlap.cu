@@ -102,6 +102,7 @@ static int inner_scratch(int dev, size_t part_len, size_t cnt_len, InnerScratch*
         s.cnt_len = 0;
         KG_CUDA(cudaMalloc(&s.cnt, sizeof(unsigned) * cnt_len));
         KG_CUDA(cudaMemset(s.cnt, 0, sizeof(unsigned) * cnt_len));
+        KG_CUDA(uploads_done());
         s.cnt_len = cnt_len;
     }
     *out = &s;

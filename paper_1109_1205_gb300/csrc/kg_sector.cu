@@ -62,6 +62,7 @@ static int upload_binomials() {
         for (int n = 0; n <= kMaxL; ++n)
             for (int k = 0; k <= kMaxL; ++k) tab[n][k] = (uint32_t)host_binom(n, k);
         cudaError_t e = cudaMemcpyToSymbol(c_binom, tab, sizeof tab);
+        if (e == cudaSuccess) e = uploads_done();
         if (e != cudaSuccess) status = cuda_fail(e, "binomial table upload", __FILE__, __LINE__);
     });
     return status;
@@ -317,7 +318,11 @@ int sector_build(int L, int nu, int nd, const double* h_re, const double* h_im, 
         cudaError_t e = cudaMalloc(&d_hnz, sizeof(uint32_t) * kMaxL);
         if (e != cudaSuccess) return fail(cuda_fail(e, "cudaMalloc", __FILE__, __LINE__));
     }
-    cudaMemcpy(d_hnz, hnz.data(), sizeof(uint32_t) * kMaxL, cudaMemcpyHostToDevice);
+    if (cudaMemcpy(d_hnz, hnz.data(), sizeof(uint32_t) * kMaxL, cudaMemcpyHostToDevice) != cudaSuccess ||
+        uploads_done() != cudaSuccess) {
+        cudaFree(d_hnz);
+        return fail(cuda_fail(cudaGetLastError(), "hopping mask upload", __FILE__, __LINE__));
+    }
     rc = build_spin(s->up, L, nu, d_hnz, eps_up.data(), s->stream);
     if (rc == KG_OK) rc = build_spin(s->dn, L, nd, d_hnz, eps_dn.data(), s->stream);
     cudaFree(d_hnz);
@@ -329,8 +334,10 @@ int sector_build(int L, int nu, int nd, const double* h_re, const double* h_im, 
         set_error("device allocation of sector tables failed");
         return fail(KG_ENOMEM);
     }
-    cudaMemcpy(s->hamp, hamp.data(), sizeof(double2) * L * L, cudaMemcpyHostToDevice);
-    cudaMemcpy(s->Utab, utab.data(), sizeof(double) * utab.size(), cudaMemcpyHostToDevice);
+    if (cudaMemcpy(s->hamp, hamp.data(), sizeof(double2) * L * L, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(s->Utab, utab.data(), sizeof(double) * utab.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        uploads_done() != cudaSuccess)
+        return fail(cuda_fail(cudaGetLastError(), "sector table upload", __FILE__, __LINE__));
     if (cudaMalloc(&s->diag, sizeof(double) * s->d) != cudaSuccess) {
         cudaGetLastError();
         set_error("device allocation of the diagonal table failed (%lld states)", s->d);
