@@ -519,6 +519,17 @@ __device__ __forceinline__ int block_max_int(int v, int* sm) {
     return m;
 }
 
+// Block maximum of an int, for all threads.
+__device__ __forceinline__ int block_max_all(int v, int* sm) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int m = sm[0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, sm[w]);
+    __syncthreads();
+    return m;
+}
+
 // Biased exponent field of an FP64 value (0 for zero).
 __device__ __forceinline__ int exp_field(double x) {
     return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);

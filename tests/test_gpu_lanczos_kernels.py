@@ -86,6 +86,25 @@ def test_scaled_start(p2, schedule):
     assert np.max(np.abs(z * 2.0 ** -p2 - y)) < TOL
 
 
+@pytest.mark.parametrize("L,n", [(4, 2), (8, 4), (10, 5), (12, 5)])  # 1, 20, 249 and 608 blocks of exponents
+@pytest.mark.parametrize("where", [0, 0.5, 1])
+def test_hpsi_largest_component(L, n, where):
+    """H*psi of uniform hopping with one component 2^40 above the others, in
+    the first, a middle and the last block: the image of x overflows if its
+    exponent is missed.  1e-12 of the largest result: each of at most 2 L hops
+    rounds to 2^-54 of the largest component, times |U| + |T| of order one."""
+    m = W.hubbard_ring(L, 4.0, n, n)
+    x = W.random_state(W.sector_dim(L, n, n), L)
+    x[int(where * (x.size - 1))] *= 2.0 ** 40
+    xd = torch.from_numpy(x.copy()).cuda()
+    yd = torch.empty_like(xd)
+    s = kg.Sector(m)
+    s.hpsi(xd, yd, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ref = oracle.Sector(m).hpsi(x)
+    assert np.max(np.abs(yd.cpu().numpy() - ref)) < 1e-12 * np.max(np.abs(ref))
+
+
 def test_small_column_near_breakdown():
     """A start vector that spans three eigenvectors to 1e-9: the space is
     nearly invariant after three vectors, so the images' exponent bounds are
