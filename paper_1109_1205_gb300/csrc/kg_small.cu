@@ -94,8 +94,11 @@ __device__ __forceinline__ unsigned cluster_size() {
 }
 // Barrier of the cluster; shared, distributed shared and global writes before
 // it are visible to the cluster's threads after it.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 __device__ __forceinline__ void remote_store(const void* p, unsigned rank, unsigned long long a, unsigned long long b) {
     unsigned addr;
@@ -211,6 +214,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
                                                               int M, int finish) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SmallShared sh;
+    // a block's shared memory may be written by another block only once it has
+    // started: waited for before the first remote_store
+    cluster_arrive();
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
     const int b = cols[blockIdx.x / C];
     const ColDesc D = desc[b];
@@ -284,6 +290,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
             ed = max(ed, exp_field(dg[q]));
         }
     }
+    cluster_wait();  // every block of the cluster runs
     if (posts) {
         em = __reduce_max_sync(0xffffffffu, em);
         ed = __reduce_max_sync(0xffffffffu, ed);
