@@ -655,12 +655,14 @@ __global__ void __launch_bounds__(IntDots<NK>::threads, 2) k_reorth_dots_int(con
             ok = ok && mbar_wait(full + t % S, (unsigned)((t / S) & 1));
             int4* img = reinterpret_cast<int4*>(dyn + (t % S) * P::kStage) + kb * T;
             const int n = min(T, len - t * T), base = (r & 1) * kThreads + (t * T) % kThreads;
-            if (any_fresh)  // re-made images replace what was copied (each thread its own elements)
+            if (any_fresh) {  // re-made images replace what was copied (each thread its own elements)
                 for (int k = 0; k < kn; ++k)
                     for (int e = tl; fresh_s[kb + k] && e < n; e += TG) {
                         const size_t at = (size_t)(k0 + kb + k) * d + e0 + (size_t)t * T + e;
                         img[k * T + e] = D.I[at] = fix_image(D.V[at], ek_s[kb + k]);
                     }
+                proxy_fence();  // ordinary stores to a stage that the next bulk copy fills again
+            }
 #pragma unroll 2
             for (int e = tl; e < n; e += TG) {
                 const int4 u = ua[base + e];

@@ -28,3 +28,14 @@ def test_cluster_runs_before_its_shared_memory_is_written():
     k = body(source("kg_small.cu"), r"k_small_step\(")
     barrier = min(i for i in (k.find("cluster_wait("), k.find("cluster_sync(")) if i >= 0)
     assert barrier < k.index("remote_store("), "remote store before the first cluster barrier"
+
+
+def test_rewritten_stages_are_fenced_before_they_are_handed_back():
+    """Images re-made in place are ordinary stores to a stage that a bulk copy
+    (the asynchronous proxy) fills next: a proxy fence has to stand between
+    them and the arrival that hands the stage back."""
+    k = body(source("kg_krylov.cu"), r"k_reorth_dots_int\(")
+    store = k.index("img[k * T + e] =")
+    back = k.index("mbar_arrive(empty", store)
+    assert "proxy_fence(" in k[store:back]
+    assert "fence.proxy.async" in body(source("kg_internal.h"), r"void proxy_fence\(")
