@@ -790,8 +790,8 @@ int green_equilibrium_vjp(kg_sector* s, const int* orb, int n_orb, double dt, in
     }
     // propagation states are checked for NaN/Inf by the Lanczos kernels
     if (rc == KG_OK && NC > 0) {
-        std::vector<ColScalars> h(NC);
-        if (cudaMemcpy(h.data(), KB.cs, sizeof(ColScalars) * NC, cudaMemcpyDeviceToHost) != cudaSuccess) rc = KG_ECUDA;
+        std::vector<ColScalars> h;
+        rc = read_scalars(KB, h, st);
         for (auto& c : h)
             if (rc == KG_OK) rc = column_rc(c.status, "the adjoint sweep");
     }

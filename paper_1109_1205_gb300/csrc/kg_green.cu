@@ -402,11 +402,7 @@ static int green_eq_batch(kg_sector* const* sv, int n_inst, const int* orb, int 
          cudaStreamSynchronize(st) != cudaSuccess))
         rc = cuda_fail(cudaGetLastError(), "overlap readback", __FILE__, __LINE__);
     std::vector<ColScalars> hcs;
-    if (rc == KG_OK) {
-        hcs.resize(K.B);
-        if (cudaMemcpy(hcs.data(), K.cs, sizeof(ColScalars) * K.B, cudaMemcpyDeviceToHost) != cudaSuccess)
-            rc = KG_ECUDA;
-    }
+    if (rc == KG_OK) rc = read_scalars(K, hcs, st);
     if (rc == KG_OK) {
         for (auto& g : G) {
             int bad = KG_OK;
@@ -1365,15 +1361,15 @@ static int block_row(kg_keldysh* X, KBlock& B, int k, cudaStream_t st) {
     return KG_OK;
 }
 
-static int block_status_of(Krylov& K, const char* what) {
-    std::vector<ColScalars> h(K.B);
-    KG_CUDA(cudaMemcpy(h.data(), K.cs, sizeof(ColScalars) * K.B, cudaMemcpyDeviceToHost));
+static int block_status_of(Krylov& K, const char* what, cudaStream_t st) {
+    std::vector<ColScalars> h;
+    KG_TRY(read_scalars(K, h, st));
     for (auto& c : h)
         KG_TRY(column_rc(c.status, what));
     return KG_OK;
 }
 
-static int block_status(KBlock& B) { return block_status_of(B.K, "step (iii)"); }
+static int block_status(KBlock& B, cudaStream_t st) { return block_status_of(B.K, "step (iii)", st); }
 
 // Writes this block's part of G(t_k, t_l) for every stored k, l.
 static void block_assemble(kg_keldysh* X, KBlock& B, const std::vector<std::complex<double>>& Gm, double* G) {
@@ -1547,7 +1543,7 @@ int keldysh_create(kg_sector* ini, kg_sector* fin, const int* orb, int n_orb, do
             if (rc == KG_OK) rc = put(k, K.vec(0, 0));
         }
         if (rc == KG_OK) rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : KG_ECUDA;
-        if (rc == KG_OK) rc = block_status_of(K, "step (ii)");
+        if (rc == KG_OK) rc = block_status_of(K, "step (ii)", st);
         R.release();
         krylov_free(K);
         cudaFree(work);
@@ -1595,7 +1591,7 @@ int keldysh_row(kg_keldysh* X, int k, double* G_les_kk, double* G_gtr_kk) {
                  cudaSuccess ||
              cudaStreamSynchronize(st) != cudaSuccess))
             rc = cuda_fail(cudaGetLastError(), "row readback", __FILE__, __LINE__);
-        if (rc == KG_OK) rc = block_status(B);
+        if (rc == KG_OK) rc = block_status(B, st);
         if (!X->keep_krylov) block_release_krylov(B);
         if (!X->keep_stores) block_release(B);
         if (rc != KG_OK) return rc;
@@ -1703,7 +1699,7 @@ int green_keldysh(kg_sector* ini, kg_sector* fin, const int* orb, int n_orb, dou
         rc = block_prepare(X, B, st, n_t, planes);
         for (int k = 0; rc == KG_OK && k < n_t; ++k) rc = block_row(X, B, k, st);
         if (rc == KG_OK) rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : KG_ECUDA;
-        if (rc == KG_OK) rc = block_status(B);
+        if (rc == KG_OK) rc = block_status(B, st);
         // the workspace goes before the Gram, which needs its own scratch
         block_release_krylov(B);
         std::vector<std::complex<double>> Gm;
@@ -1845,7 +1841,7 @@ static int pair_vectors(kg_sector* fin, kg_sector* s1, kg_sector* s2, FourOp A, 
                 }
             }
             if (rc == KG_OK) rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : KG_ECUDA;
-            if (rc == KG_OK) rc = block_status_of(K, "the four-time sweeps");
+            if (rc == KG_OK) rc = block_status_of(K, "the four-time sweeps", st);
         }
         R.release();
         krylov_free(K);
@@ -1873,7 +1869,7 @@ static int pair_vectors(kg_sector* fin, kg_sector* s1, kg_sector* s2, FourOp A, 
             rc = cuda_fail(cudaGetLastError(), "four-time columns out", __FILE__, __LINE__);
     }
     if (rc == KG_OK) rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : KG_ECUDA;
-    if (rc == KG_OK) rc = block_status_of(K, "the four-time back-propagation");
+    if (rc == KG_OK) rc = block_status_of(K, "the four-time back-propagation", st);
     R.release();
     krylov_free(K);
     return rc;
@@ -1960,7 +1956,7 @@ int green_four_time(kg_sector* ini, kg_sector* fin, const int* ops, double dt, i
                 rc = cuda_fail(cudaGetLastError(), "Phi(t_k)", __FILE__, __LINE__);
         }
         if (rc == KG_OK) rc = cudaStreamSynchronize(st) == cudaSuccess ? KG_OK : KG_ECUDA;
-        if (rc == KG_OK) rc = block_status_of(K, "step (ii)");
+        if (rc == KG_OK) rc = block_status_of(K, "step (ii)", st);
         R.release();
         krylov_free(K);
     }

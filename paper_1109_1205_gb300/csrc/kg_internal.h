@@ -337,6 +337,9 @@ struct StepRunner {
     void release();
 };
 
+// The columns' scalars on the host, after everything queued on `st`, the stream
+// whose kernels write them.
+int read_scalars(const Krylov& K, std::vector<ColScalars>& h, cudaStream_t st);
 // KG_OK, or the status a column's kernels reported (non-finite value, device
 // wait run out) with the error message set.
 int column_rc(int status, const char* what);

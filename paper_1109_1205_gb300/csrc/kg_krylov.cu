@@ -1680,6 +1680,13 @@ int enqueue_step(Krylov& K, int reorth, cudaStream_t st) {
     return launch_combine(K, st);
 }
 
+int read_scalars(const Krylov& K, std::vector<ColScalars>& h, cudaStream_t st) {
+    h.resize(K.B);
+    KG_CUDA(cudaMemcpyAsync(h.data(), K.cs, sizeof(ColScalars) * K.B, cudaMemcpyDeviceToHost, st));
+    KG_CUDA(cudaStreamSynchronize(st));
+    return KG_OK;
+}
+
 int column_rc(int status, const char* what) {
     if (status == KG_ENUMERIC) set_error("non-finite value during %s", what);
     else if (status == KG_ETIMEOUT) set_error("a bounded device wait ran out during %s", what);

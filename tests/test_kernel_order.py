@@ -39,3 +39,12 @@ def test_rewritten_stages_are_fenced_before_they_are_handed_back():
     back = k.index("mbar_arrive(empty", store)
     assert "proxy_fence(" in k[store:back]
     assert "fence.proxy.async" in body(source("kg_internal.h"), r"void proxy_fence\(")
+
+
+def test_scalars_are_read_on_the_stream_that_writes_them():
+    """The kernels run on non-blocking streams, which a synchronous cudaMemcpy
+    (the legacy stream) does not wait for: a status read that way can miss
+    what the last steps report."""
+    for name in sorted(os.listdir(CSRC)):
+        for call in re.findall(r"\bcudaMemcpy\s*\(([^;]*)", source(name)):
+            assert not ("DeviceToHost" in call and re.search(r"\bcs\b", call)), (name, call)
