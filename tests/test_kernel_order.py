@@ -1,5 +1,5 @@
-"""Orderings that the kernels need and no run can show to be missing, read from
-the sources (comments removed)."""
+"""Orderings that the kernels need and no run can show to be missing, and one
+cost that no result shows, read from the sources (comments removed)."""
 import os
 import re
 
@@ -48,3 +48,11 @@ def test_scalars_are_read_on_the_stream_that_writes_them():
     for name in sorted(os.listdir(CSRC)):
         for call in re.findall(r"\bcudaMemcpy\s*\(([^;]*)", source(name)):
             assert not ("DeviceToHost" in call and re.search(r"\bcs\b", call)), (name, call)
+
+
+def test_no_constant_table_in_a_shared_header():
+    """A __constant__ table in a header gives every module that includes it a
+    constant bank, which each launch of each of its kernels pays for."""
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith(".h"):
+            assert "__constant__" not in source(name), name
