@@ -806,9 +806,6 @@ struct Tridiag {
 // lanes or one), and the scalars between two barriers are one warp's work:
 // powers of two, exponent bounds and FP32 roundings are therefore made on the
 // integer pipe, and what can wait is computed beside the other warps' work.
-__device__ __forceinline__ double pow2i(int e) {
-    return (unsigned)(e + 1022) < 2046u ? __longlong_as_double((long long)(e + 1023) << 52) : ldexp(1.0, e);
-}
 // x 2^de without an FP64 operation where x and the result are normal.
 __device__ __forceinline__ double mul_pow2(double x, int de) {
     const int e = exp_field(x);

@@ -202,7 +202,7 @@ struct SmallShared {
     SecView S;
     double sj, cprev, aj, araw, hre;
     float r0;
-    int Ew, Eu, Ef, m_eff, status, loose, n32, n64;
+    int Ew, Eu, Ef, m_eff, status, loose, n32, n64, ec;
     int any64[8], eh[8];  // per warp of coefficients
     int E0, Ed, Ea;
 };
@@ -717,6 +717,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+        // the FP32 terms in units of 2^(ec - 1023), so that none vanishes or overflows
+        const int ec = exp_field(cmax);
         int a32 = 0, a64 = 0;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -726,8 +728,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
             const unsigned before = (1u << lane) - 1u;
             if (small) {
                 const int q = a32 + __popc(ms & before);
-                const double f = pow2i(eimg[k] - 1050);
-                coef32[q] = make_float2(f64_to_f32_near(c[r].x * f), f64_to_f32_near(c[r].y * f));
+                const int de = eimg[k] - 1050 + 1023 - ec;
+                coef32[q] = make_float2(f64_to_f32_near(mul_pow2(c[r].x, de)), f64_to_f32_near(mul_pow2(c[r].y, de)));
                 idx32[q] = (short)k;
             } else if (k < m) {
                 const int q = a64 + __popc(in & ~ms & before);
@@ -740,6 +742,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
         if (lane == 0) {
             sh.n32 = a32;
             sh.n64 = a64;
+            sh.ec = ec;
         }
     }
     __syncthreads();
@@ -778,8 +781,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
             cx = fmaf(c.x, vx, fmaf(-c.y, vy, cx));
             cy = fmaf(c.x, vy, fmaf(c.y, vx, cy));
         }
-        u.x += (double)cx;
-        u.y += (double)cy;
+        u.x += mul_pow2(f32_to_f64_int(cx), sh.ec - 1023);
+        u.y += mul_pow2(f32_to_f64_int(cy), sh.ec - 1023);
         D.out[e0 + i] = u;
         w[q] = u;
         nrm = fma(u.x, u.x, fma(u.y, u.y, nrm));

@@ -1,0 +1,52 @@
+"""Start vectors and Hamiltonians far from one: what the kernels keep in FP32
+may neither vanish nor overflow.
+
+Everything is scaled by powers of two (x by 2^p; H by 2^q and the step by
+2^-q), so exact arithmetic gives the unscaled result times 2^p, and FP64 at
+these exponents the same roundings.  Tolerance 1e-13 on unit vectors: a term may
+move between its FP32 and FP64 sums, which changes a few roundings of 1e-16
+in each of the 40 to 80 Lanczos vectors of a run, while a lost FP32 term of
+the combination is 1e-13 to 1e-10 of the result.
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1109_1205_gb300 as kg  # noqa: E402
+
+TOL = 1e-13
+
+
+def model(name, q=0):
+    if name == "star":
+        rng = np.random.default_rng(6)
+        m = W.siam_star(-1.5, 3.0, rng.uniform(-3, 3, 5), rng.uniform(0.2, 1.0, 5), 3, 3)
+    elif name == "ring":
+        m = W.hubbard_ring(8, 4.0, 4, 4)
+    else:
+        L = 8 if name == "random8" else 9
+        m = W.random_model(L, 4, 4, seed=20, complex_hopping=True)
+    return dict(m, h=np.asarray(m["h"]) * 2.0 ** q, eps=np.asarray(m["eps"]) * 2.0 ** q,
+                U=np.asarray(m["U"]) * 2.0 ** q)
+
+
+def run(name, p, q, schedule, M=20):
+    s = kg.Sector(model(name, q))
+    x = W.random_state(s.dim, 20)
+    xd = torch.from_numpy(x * 2.0 ** p).cuda()
+    s.propagate(xd, 0.02 * 2.0 ** -q, 2, kg.kg_opts_default(M=M, schedule=schedule))
+    torch.cuda.synchronize()
+    return xd.cpu().numpy() * 2.0 ** -p
+
+
+# small columns (one cluster per column) of each kind of hop sum
+@pytest.mark.parametrize("name", ["star", "ring", "random8"])
+@pytest.mark.parametrize("p", [-400, -130, -100, -61, 61, 130, 161, 400])
+def test_scaled_start_of_a_small_column(name, p):
+    assert np.max(np.abs(run(name, p, 0, 0) - run(name, 0, 0, 0))) < TOL
