@@ -445,9 +445,17 @@ int green_equilibrium_batched(kg_sector* const* s, int n_inst, const int* orb, i
 // this GPU, or sixteen 32 x 32 -> 64 bit integer ones of 52-bit fixed-point
 // images (kg_krylov.cu, the exact dots), half a cycle.  So the vectors are
 // converted on their own largest exponents when a tile is staged, the products
-// are summed exactly and go to FP64 every kGramFlush elements.  The images'
-// rounding, 2^-53 of a vector's largest component per element, adds at most
-// 2^-53 ||x|| ||y|| to a sum, less than the rounding of an FP64 sum.
+// are summed exactly and go to FP64 every kGramFlush elements.
+//
+// What an image leaves off, up to 2^-53 of its vector's largest component in
+// every element, could add up to sqrt(d) 2^-53 ||x|| ||y|| (a vector with one
+// dominant component against one that lives on the others), where FP64 products
+// lose nothing.  It is therefore kept in FP32 beside the image, and the two
+// cross products with the other vector are added to the integer sums: eight
+// FP32 multiply-adds per complex product, beside sixteen integer ones that take
+// eight times as long.  What is dropped then is 2^-76 of the product of the
+// largest components, and the sum over the slabs carries its rounding along,
+// so an entry is as exact as its slabs' few roundings.
 //
 // A thread takes 2 x 2 outputs {I, I + H} x {J, J + H} of a tile, H half its
 // rows, so that neighbouring lanes read neighbouring rows; a diagonal tile
@@ -472,10 +480,32 @@ __global__ void __launch_bounds__(kThreads) k_gram_exp(const double2* __restrict
     if (threadIdx.x == 0) atomicMax(emax + blockIdx.y, m);
 }
 
+// The part of x on a bound's exponent field E that fix52(x, E) rounds off, in
+// half units of the image (|result| <= 1), to FP32 precision.
+__device__ __forceinline__ float fix52_rest(double x, int E) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ffull), t = E + 1 - e;  // the image drops t bits
+    if (e == 0 || t > 140) return 0.0f;
+    const long long m = (long long)((b & 0xfffffffffffffull) | 0x10000000000000ull);
+    long long rem = m;
+    int sh = 22;  // to 31 bits: all 53 bits of x are left off
+    if (t <= 53) {
+        rem = m - (((m + (1ll << (t - 1))) >> t) << t);
+        sh = max(0, t - 31);
+    }
+    const float v = (float)(int)(rem >> sh) * __int_as_float((sh - (t - 1) + 127) << 23);
+    return (b >> 63) ? -v : v;
+}
+
+constexpr int kGramBuf = 2 * kGT * (kGK + 1);  // staged elements, rows 16 bytes apart mod 128
+constexpr size_t kGramSmem = 2 * kGramBuf * (sizeof(int4) + sizeof(float4));
+
 __global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, int nv, int d, int ntile, int slab,
                                                  const int2* __restrict__ tiles, const int* __restrict__ emax,
                                                  double2* __restrict__ part) {
-    __shared__ int4 st[2][2 * kGT][kGK + 1];  // rows of the two operands, 16-byte stride between rows mod 128
+    extern __shared__ __align__(16) unsigned char dyn[];
+    int4* const st = reinterpret_cast<int4*>(dyn);  // [2][rows of the two operands][kGK + 1] images
+    float4* const sr = reinterpret_cast<float4*>(st + 2 * kGramBuf);  // what they leave off, their upper halves
     const int2 tl = tiles[blockIdx.x];
     const bool diag = tl.x == tl.y;
     const int p0 = tl.x * kGT, q0 = tl.y * kGT;
@@ -516,7 +546,11 @@ __global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, 
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int r = r0 + 16 * u;
-            if (r < rows) st[b][r][c] = fix_image(nx[u], ex[u]);
+            if (r >= rows) continue;
+            const int at = b * kGramBuf + r * (kGK + 1) + c;
+            const int4 f = fix_image(nx[u], ex[u]);
+            st[at] = f;
+            sr[at] = make_float4(fix52_rest(nx[u].x, ex[u]), fix52_rest(nx[u].y, ex[u]), (float)(f.x + (f.y >> 25)), (float)(f.z + (f.w >> 25)));
         }
     };
     double2 acc[2][2];
@@ -548,8 +582,8 @@ __global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, 
     for (int i0 = i_begin, b = 0; i0 < i_end; i0 += kGK, b ^= 1) {
         if (i0 + kGK < i_end) load(i0 + kGK);
         if (use) {
-            const int4* A = &st[b][I][0];
-            const int4* B = &st[b][(diag ? 0 : kGT) + J][0];
+            const int oa = b * kGramBuf + I * (kGK + 1), ob = b * kGramBuf + ((diag ? 0 : kGT) + J) * (kGK + 1);
+            const int4 *A = st + oa, *B = st + ob;
             const int ah = Hp * (kGK + 1), bh = Hq * (kGK + 1);
 #pragma unroll 2
             for (int k = 0; k < kGK; ++k) {
@@ -560,6 +594,31 @@ __global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, 
                 cdot_fix(a1, b0, m0, re[1][0], im[1][0]);
                 cdot_fix(a1, b1, m1, re[1][1], im[1][1]);
             }
+            // half units times upper halves (rounded to 2^26 units): the cross
+            // products in units of 2^26 after halving, at most 2^31 over the step
+            // (where the conversion saturates)
+            const float4 *Ar = sr + oa, *Br = sr + ob;
+            float cr[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, ci[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll 2
+            for (int k = 0; k < kGK; ++k) {
+                const float4 a[2] = {Ar[k], Ar[ah + k]}, q[2] = {Br[k], Br[bh + k]};
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        cr[x][y] = fmaf(a[x].x, q[y].z, fmaf(a[x].z, q[y].x, cr[x][y]));
+                        cr[x][y] = fmaf(a[x].y, q[y].w, fmaf(a[x].w, q[y].y, cr[x][y]));
+                        ci[x][y] = fmaf(a[x].x, q[y].w, fmaf(a[x].z, q[y].y, ci[x][y]));
+                        ci[x][y] = fmaf(-a[x].y, q[y].z, fmaf(-a[x].w, q[y].x, ci[x][y]));
+                    }
+            }
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    re[x][y][1] += __float2int_rn(0.5f * cr[x][y]);
+                    im[x][y][1] += __float2int_rn(0.5f * ci[x][y]);
+                }
             held += kGK;
             if (held == kGramFlush) {
                 flush();
@@ -578,27 +637,46 @@ __global__ void __launch_bounds__(256, 2) k_gram(const double2* __restrict__ X, 
         for (int y = 0; y < 2; ++y) out[(I + x * Hp) * kGT + J + y * Hq] = acc[x][y];
 }
 
-__global__ void k_gram_reduce(const double2* part, int nz, int ntile, const int2* tiles, const int* emax, int nv,
-                              double2* G) {
-    const int e = threadIdx.x + blockDim.x * blockIdx.y;
-    if (e >= kGT * kGT) return;
+// (s, c) += (v, w) with s's rounding error added to c (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(double& s, double& c, double v, double w) {
+    const double t = s + v, z = t - s;
+    c += w + ((s - (t - z)) + (v - z));
+    s = t;
+}
+
+// The slabs' sums and their units: 32 entries per block, the slabs split over
+// its eight warps, in a fixed order.
+__global__ void __launch_bounds__(256) k_gram_reduce(const double2* part, int nz, int ntile, const int2* tiles,
+                                                     const int* emax, int nv, double2* G) {
+    __shared__ double sm[8][4][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = 32 * blockIdx.y + lane;
     const int2 tl = tiles[blockIdx.x];
     const bool diag = tl.x == tl.y;
     const int Hp = (min(kGT, nv - tl.x * kGT) + 1) / 2, Hq = (min(kGT, nv - tl.y * kGT) + 1) / 2;
     const int r = e / kGT, c = e % kGT, p = tl.x * kGT + r, q = tl.y * kGT + c;
-    if (r >= 2 * Hp || c >= 2 * Hq || p >= nv || q >= nv) return;
-    if (diag && r % Hp > c % Hp) return;         // not computed
-    if (diag && r == c + Hp) return;             // its mirror is
-    double2 s = make_double2(0.0, 0.0);
-    for (int z = 0; z < nz; ++z) {
-        const double2 v = part[((size_t)z * ntile + blockIdx.x) * kGT * kGT + e];
-        s.x += v.x;
-        s.y += v.y;
+    // in a diagonal tile one entry of each mirrored pair is computed
+    const bool take = r < 2 * Hp && c < 2 * Hq && p < nv && q < nv && !(diag && (r % Hp > c % Hp || r == c + Hp));
+    double2 s = make_double2(0.0, 0.0), t = s;
+    if (take)
+        for (int z = warp; z < nz; z += 8) {
+            const double2 v = part[((size_t)z * ntile + blockIdx.x) * kGT * kGT + e];
+            two_sum(s.x, t.x, v.x, 0.0);
+            two_sum(s.y, t.y, v.y, 0.0);
+        }
+    sm[warp][0][lane] = s.x;
+    sm[warp][1][lane] = t.x;
+    sm[warp][2][lane] = s.y;
+    sm[warp][3][lane] = t.y;
+    __syncthreads();
+    if (warp != 0 || !take) return;
+    for (int w = 1; w < min(8, nz); ++w) {
+        two_sum(s.x, t.x, sm[w][0][lane], sm[w][1][lane]);
+        two_sum(s.y, t.y, sm[w][2][lane], sm[w][3][lane]);
     }
-    // units of the images; a non-finite vector has none
+    // a non-finite vector has no units
     const double f = emax[p] == 2047 || emax[q] == 2047 ? nan("") : ldexp(1.0, emax[p] + emax[q] - 2096);
-    s.x *= f;
-    s.y = p == q ? 0.0 * f : s.y * f;
+    s.x = (s.x + t.x) * f;
+    s.y = p == q ? 0.0 * f : (s.y + t.y) * f;
     G[(size_t)p * nv + q] = s;
     G[(size_t)q * nv + p] = make_double2(s.x, -s.y);
 }
@@ -628,6 +706,7 @@ struct GramPlan {
             set_error("Gram scratch of %d vectors", nv);
             return KG_ENOMEM;
         }
+        KG_CUDA(cudaFuncSetAttribute((const void*)k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem));
         KG_CUDA(cudaMemcpy(tiles, v.data(), sizeof(int2) * ntile, cudaMemcpyHostToDevice));
         KG_CUDA(uploads_done());
         return KG_OK;
@@ -637,8 +716,8 @@ struct GramPlan {
         KG_CUDA(cudaMemsetAsync(emax, 0, sizeof(int) * nv, st));
         const int be = std::max(1, std::min((d + kThreads - 1) / kThreads, (nsm * 8 + nv - 1) / nv));
         k_gram_exp<<<dim3(be, nv), kThreads, 0, st>>>(X, d, emax);
-        k_gram<<<dim3(ntile, nz), 256, 0, st>>>(X, nv, d, ntile, slab, tiles, emax, part);
-        k_gram_reduce<<<dim3(ntile, kGT * kGT / 256), 256, 0, st>>>(part, nz, ntile, tiles, emax, nv, G);
+        k_gram<<<dim3(ntile, nz), 256, kGramSmem, st>>>(X, nv, d, ntile, slab, tiles, emax, part);
+        k_gram_reduce<<<dim3(ntile, kGT * kGT / 32), 256, 0, st>>>(part, nz, ntile, tiles, emax, nv, G);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch", __FILE__, __LINE__);
         count_launch(3);
