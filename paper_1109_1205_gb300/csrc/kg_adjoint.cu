@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(kGradThreads) k_lincomb(const ColDesc* desc, c
             const double2* ck = cq + (size_t)b * NT * Mcap + k;
             bool small = false;
             if (k < m) {
-                // both norms within 2^-60 .. 2^60: the FP32 copies neither overflow nor vanish
+                // both norms and their product (the coefficients) within 2^-60 .. 2^60: the
+                // FP32 copies do not overflow, nor vanish above 2^-64 of the result
                 const double sk = C->scale[k];
                 const int es = exp_field(sk);
                 float big = 0.0f;
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(kGradThreads) k_lincomb(const ColDesc* desc, c
                     const double2 v = ck[(size_t)t * Mcap];
                     big = fmaxf(big, scaled_abs(v.x, 0) + scaled_abs(v.y, 0));
                 }
-                small = (unsigned)(es - 963) <= 120u && (unsigned)(eb - 963) <= 120u &&
+                small = (unsigned)(es - 963) <= 120u && (unsigned)(eb - 963) <= 120u && (unsigned)(es + eb - 1986) <= 120u &&
                         big < 1e-10f * (scaled_abs(beta0, 0) * scaled_abs(sk, 0));
             }
             const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, small);

@@ -835,8 +835,11 @@ __global__ void __launch_bounds__(kThreads) k_update(const ColDesc* desc, const 
                 const int de = C->emax[k] - ew;
                 r += scaled_abs(c.x, de) + scaled_abs(c.y, de);
             }
-            // |h_k| for the unit vector v_k; a start vector of extreme norm (c or its FP32 copy out of range) stays in FP64
-            const bool small = scaled_abs(h.x, 0) + scaled_abs(h.y, 0) < (float)kSmallCoef && (unsigned)(es - 963) <= 120u;
+            // |h_k| for the unit vector v_k.  In FP64 where the FP32 copy of V_k leaves
+            // FP32's range, or where c = s_k h_k or the sum could vanish (below
+            // 2^-126) while they count beside w (above 2^-64 of its bound)
+            const bool small = scaled_abs(h.x, 0) + scaled_abs(h.y, 0) < (float)kSmallCoef &&
+                               (unsigned)(es - 963) <= 120u && es + ew >= 1983 && ew >= 960;
             const unsigned in = __ballot_sync(0xffffffffu, k < nk), ms = __ballot_sync(0xffffffffu, k < nk && small);
             const unsigned before = (1u << lane) - 1u;
             if (k < nk && small) {
@@ -1440,13 +1443,17 @@ __global__ void __launch_bounds__(kThreads) k_combine(const ColDesc* desc, const
 #pragma unroll
         for (int o_ = 16; o_ > 0; o_ >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o_));
         int a64 = 0, a32 = 0;
-        // norms within 2^-60 .. 2^60: the FP32 copies and coefficients neither overflow nor vanish
-        const bool in32 = V32 && (unsigned)(exp_field(cmax) - 963) <= 120u;
+        // norms, and their product (the coefficients), within 2^-60 .. 2^60: the FP32
+        // copies and coefficients do not overflow, nor vanish above 2^-64 of the result
+        const int ec = exp_field(cmax);
+        const bool in32 = V32 && (unsigned)(ec - 963) <= 120u;
         for (int k0 = 0; k0 < m; k0 += 32) {
             const int k = k0 + lane;
             const double2 c = k < m ? C->c[k] : make_double2(0.0, 0.0);
             const double sk = k < m ? C->scale[k] : 0.0;
-            const bool small = in32 && (unsigned)(exp_field(sk) - 963) <= 120u && (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
+            const int es = exp_field(sk);
+            const bool small = in32 && (unsigned)(es - 963) <= 120u && (unsigned)(ec + es - 1986) <= 120u &&
+                               (fabs(c.x) + fabs(c.y)) < 1e-10 * cmax * sk;
             const unsigned in = __ballot_sync(0xffffffffu, k < m), ms = __ballot_sync(0xffffffffu, k < m && small);
             const unsigned before = (1u << lane) - 1u;
             if (k < m && small) {

@@ -50,3 +50,11 @@ def run(name, p, q, schedule, M=20):
 @pytest.mark.parametrize("p", [-400, -130, -100, -61, 61, 130, 161, 400])
 def test_scaled_start_of_a_small_column(name, p):
     assert np.max(np.abs(run(name, p, 0, 0) - run(name, 0, 0, 0))) < TOL
+
+
+@pytest.mark.parametrize("name,schedule", [("star", 0), ("ring", 0), ("random8", 0),
+                                           ("random9", 2), ("random9", 4)])  # and the streaming kernels
+@pytest.mark.parametrize("p,q", [(0, -70), (0, -40), (0, 58), (-58, 58), (-58, 55), (-60, 53), (58, -58), (0, 130),
+                                 (30, -130)])
+def test_scaled_hamiltonian(name, schedule, p, q):
+    assert np.max(np.abs(run(name, p, q, schedule) - run(name, 0, 0, schedule))) < TOL
