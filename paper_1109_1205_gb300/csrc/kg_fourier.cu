@@ -27,7 +27,7 @@
 // e^{i omega t_c} F_c(omega), F_c(omega) = sum_q g_q e^{i omega (t_q - t_c)},
 // and F_c has only frequencies up to B dt / 2 as a function of omega: on a
 // window of omega of width D it is a polynomial of degree K - 1 through its
-// values at K Chebyshev nodes up to 2 (D B dt / 8)^K / K!, below 1e-17 of
+// values at K Chebyshev nodes up to 2 (D B dt / 8)^K / K!, below 2e-17 of
 // sum |g_q| for K = 24 and D B dt <= 15.2.  So the sums are taken at the nodes
 // only (168 of them instead of 4,001 frequencies on the paper's grid with
 // B = 512), two real multiply-adds per sample, node and part, the cosines and
@@ -308,9 +308,12 @@ static FtPlan ft_plan(int n_series, int n_t, double dt, const double* omega, int
         FtPlan P;
         P.B = B;
         P.W = std::max(1, (int)std::ceil(width));
-        // one frequency (or several equal ones): a window around it
-        P.D = hi > lo ? (hi - lo) / P.W : kFtPhase / T;
-        P.omega0 = hi > lo ? lo : lo - 0.5 * P.D;
+        // a single window is as wide as it may be, around its frequencies: equal or
+        // nearly equal ones would otherwise have nodes that FP64 cannot tell apart
+        P.D = P.W > 1 ? (hi - lo) / P.W : kFtPhase / T;
+        P.omega0 = P.W > 1 ? lo : 0.5 * lo + 0.5 * hi - 0.5 * P.D;
+        // as when the frequencies are that large themselves
+        if (P.D < 0x1p-40 * std::max(std::fabs(lo), std::fabs(hi))) break;
         P.runs = (int)((n_t + (long long)B - 1) / B);
         P.groups = (P.runs + kFtGroup - 1) / kFtGroup;
         const double nodes = (double)P.W * kFtK;
