@@ -179,14 +179,14 @@ __global__ void __launch_bounds__(kFtThreads) k_ft_weights(const double* __restr
 }
 
 // cos and sin of nu_m tau_q (node m of all windows, tau_q = (q + 1/2) dt), and
-// the damping e^{-+eta tau_q} on both sides of a run's centre.
+// the damping from the run's start to the samples on both sides of its centre
+// (at most 1, so that no sample overflows).
 __global__ void __launch_bounds__(kFtThreads) k_ft_table(FtPlan P, double dt, double eta, double2* __restrict__ table,
                                                          double2* __restrict__ damp) {
     const int n = P.W * kFtK, half = P.B / 2;
     const int e = blockIdx.x * kFtThreads + threadIdx.x;
     if (e < half) {
-        const double a = eta * ((e + 0.5) * dt);
-        damp[e] = make_double2(exp(-a), exp(a));
+        damp[e] = make_double2(exp(-eta * ((half + e) * dt)), exp(-eta * ((half - 1 - e) * dt)));
     }
     if (e >= n * half) return;
     const int q = e / n, m = e - q * n, win = m / kFtK;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kFtThreads) k_ft_table(FtPlan P, double dt, do
     table[e] = make_double2(c, s);
 }
 
-// F[series][run][node] = e^{-eta t_c} sum over the run, kFtRuns runs per block,
+// F[series][run][node] = sum over the run, damped, kFtRuns runs per block,
 // one node per thread.  With a = g_+ + g_-, b = i (g_+ - g_-) of the samples at
 // t_c +- tau_q: F = sum_q cos(nu tau_q) a_q + sin(nu tau_q) b_q.
 __global__ void __launch_bounds__(kFtNodeThreads) k_ft_nodes(const double2* __restrict__ Gt, int n_t, double dt,
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kFtNodeThreads) k_ft_nodes(const double2* __re
 #pragma unroll
         for (int r = 0; r < kFtRuns; ++r)
             if (c0 + r < P.runs) {
-                const double d = exp(-eta * (((c0 + r) + 0.5) * P.B - 0.5) * dt);
+                const double d = exp(-eta * ((double)(c0 + r) * P.B * dt));
                 F[((size_t)series * P.runs + c0 + r) * nodes + m] = make_double2(d * acc[r].x, d * acc[r].y);
             }
 }
