@@ -829,7 +829,10 @@ __device__ __forceinline__ int bound_exp(float r, int base) {
     const unsigned b = __float_as_uint(r);
     return base + (int)(b >> 23) - 126 - ((b & 0x7fffffu) == 0u ? 1 : 0);
 }
-// 1 / sqrt(x) for normal x > 0: a 23-bit start and one step of third order.
+// 1 / sqrt(x) for normal x > 0.  With y near 1 / sqrt(m) and r = 1 - m y^2,
+// 1 / sqrt(m) = y (1 - r)^(-1/2) = y (1 + r / 2 + 3 r^2 / 8 + ...), the binomial
+// series.  The starting value is an FP32 reciprocal square root (|r| < 2^-20),
+// so what follows, 5 r^3 / 16, is below 2^-61.
 __device__ __forceinline__ double rsqrt3(double x) {
     // x = m 2^(2 q), m in [1, 4)
     const int e = exp_field(x) - 1023, q = e >> 1;
@@ -837,6 +840,12 @@ __device__ __forceinline__ double rsqrt3(double x) {
     const double y = f32_to_f64_int(rsqrtf(f64_to_f32_trunc(m)));
     const double r = fma(-m * y, y, 1.0);
     return mul_pow2(fma(y * r, fma(r, 0.375, 0.5), y), -q);
+}
+// sqrt(x) from r near 1 / sqrt(x): x r after one step of Newton's method,
+// q + (x - q^2) / (2 q).
+__device__ __forceinline__ double sqrt_from(double x, double r) {
+    const double q = x * r;
+    return fma(0.5 * r, fma(-q, q, x), q);
 }
 __device__ __forceinline__ int bound_exp(double r, int base) {
     int ex;
@@ -960,11 +969,10 @@ __device__ __forceinline__ void resolve_norm(const ColDesc& D, ColScalars* C, in
     const Partial t = sum_partials(D.part_n, C->n_norm, sh.sum);
     if (threadIdx.x < 32) {
         const double a = C->abase + C->hre, ref = 1e-12 * fmax(fabs(a) + C->beta[j - 1], 1e-300);
-        // b_j and 1/b_j from one reciprocal square root, b_j with its last rounding mended
+        // b_j and 1/b_j from one reciprocal square root
         const bool some = t.v > 0.0 && exp_field(t.v) != 2047;
         const double rs = some ? (exp_field(t.v) > 0 ? rsqrt3(t.v) : 1.0 / sqrt(t.v)) : 0.0;
-        const double q = t.v * rs;
-        const double b = some ? fma(0.5 * rs, fma(-q, q, t.v), q) : t.v;  // 0, infinity or NaN
+        const double b = some ? sqrt_from(t.v, rs) : t.v;  // 0, infinity or NaN
         const bool bad = exp_field(t.v) == 2047 || exp_field(a) == 2047 || (int)t.e == 2047;
         const int m = bad || !(b > ref) ? j : m_old;  // happy breakdown: K_j is invariant
         const double cp = b * C->scale[j - 1];

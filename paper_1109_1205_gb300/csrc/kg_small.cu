@@ -460,9 +460,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
     };
     double fa = 0.0, faj = 0.0;
     auto resolve_rest = [&](int j) {
-        // b_j with the last rounding of its square root mended
-        const double q = q_n2 * q_rs;
-        const double b = q_rs != 0.0 ? fma(0.5 * q_rs, fma(-q, q, q_n2), q) : 0.0;
+        const double b = q_rs != 0.0 ? sqrt_from(q_n2, q_rs) : 0.0;
         if (lane == 0) {
             if (j > 0) alpha[j - 1] = q_a;
             beta[j] = mul_pow2(b, q_e - 1064);  // beta[0]: ||V_0||
