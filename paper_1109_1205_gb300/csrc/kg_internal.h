@@ -554,7 +554,8 @@ __device__ __forceinline__ long long fix_term(double x, int E, int P, uint32_t n
 
 // v * 2^(E - 1075 - P) rounded to nearest (ties to even), assembled on the
 // integer pipe: the FP64 pipe of this GPU is the scarce one.  |v| < 2^62.
-// Falls back to FP64 arithmetic if the result would be subnormal.
+// Falls back to FP64 arithmetic if the result would be subnormal; infinite
+// above FP64's range.
 __device__ __forceinline__ double fix_to_double(long long v, int E, int P) {
     if (v == 0) return 0.0;
     const unsigned long long sgn = (unsigned long long)v & 0x8000000000000000ull;
@@ -578,6 +579,7 @@ __device__ __forceinline__ double fix_to_double(long long v, int E, int P) {
         const long long ex = (long long)E - 52 - P;
         return ex > 0 ? __ll2double_rn(v) * __longlong_as_double(ex << 52) : 0.0;
     }
+    if (be > 2046) return __longlong_as_double((long long)(sgn | 0x7ff0000000000000ull));
     return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (m & 0xfffffffffffffull)));
 }
 

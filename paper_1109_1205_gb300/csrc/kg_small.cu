@@ -435,7 +435,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
         const bool some = n2 > 0.0 && !bad;
         const double rs = some ? rsqrt3(n2) : 0.0;
         const double b = mul_pow2(n2 * rs, E - 1064), sj = mul_pow2(rs, 1064 - E);
-        const bool fin = !bad && exp_field(b) != 2047 && (j == 0 || exp_field(q_a) != 2047);
+        // norms of 2^512 and above, whose squares FP64 does not hold, are refused as
+        // by the streaming kernels: products of two scales would leave its range
+        const bool fin = !bad && exp_field(b) < 1023 + 512 && (j == 0 || exp_field(q_a) != 2047);
         int m = M;
         // happy breakdown: K_j is invariant (positive doubles compare like their bits)
         if (j == 0 ? !some : __double_as_longlong(b) <= __double_as_longlong(q_ref)) m = j;

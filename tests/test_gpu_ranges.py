@@ -58,3 +58,24 @@ def test_scaled_start_of_a_small_column(name, p):
                                  (30, -130)])
 def test_scaled_hamiltonian(name, schedule, p, q):
     assert np.max(np.abs(run(name, p, q, schedule) - run(name, 0, 0, schedule))) < TOL
+
+
+def outcome(name, p, q, schedule):
+    try:
+        return run(name, p, q, schedule)
+    except kg.KGError as e:
+        assert e.code == kg.KG_ENUMERIC
+        return None
+
+
+@pytest.mark.parametrize("name", ["star", "ring", "random8"])
+@pytest.mark.parametrize("p,q", [(500, 3), (508, 0), (520, 0), (600, 0), (1000, 3), (1015, 3), (1022, 3), (0, 500), (0, 520),
+                                 (0, 800), (0, 1010), (505, 515), (500, 500), (-500, 600)])
+def test_what_is_out_of_range_is_refused(name, p, q):
+    """Norms whose squares leave FP64's range are refused by the streaming
+    kernels (schedule = 4), and so they are for a small column; anything else
+    gives the scaled result."""
+    y, z = outcome(name, p, q, 0), outcome(name, p, q, 4)
+    assert (y is None) == (z is None)
+    if y is not None:
+        assert np.max(np.abs(y - run(name, 0, 0, 0))) < TOL
