@@ -601,7 +601,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_step(const ColDesc* des
                 const double vr = limbs_value(r0, r1), vi = limbs_value(i0, i1);
                 const double hx = f * vr, hy = f * vi;
                 if (k == j) sh.hre = hx;
-                big = !(scaled_abs(hx, 0) + scaled_abs(hy, 0) < (float)kSmallCoef);
+                // in FP64 also where the term or its factor on the upper halves (28 bits
+                // below) could vanish, below 2^-126, while the term counts beside w
+                // (above 2^-64 of it)
+                big = !(scaled_abs(hx, 0) + scaled_abs(hy, 0) < (float)kSmallCoef) || sh.Ew < 988;
                 coef32[k] = big ? make_float2(0.f, 0.f) : make_float2(f64_to_f32_near(f32 * vr), f64_to_f32_near(f32 * vi));
                 coef64[k] = make_double2(big ? fc * vr : 0.0, big ? fc * vi : 0.0);
                 // |c_k V_k| < 2^(eh - 1022)

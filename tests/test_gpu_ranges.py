@@ -11,7 +11,9 @@ the combination is 1e-13 to 1e-10 of the result.
 import numpy as np
 import pytest
 
+import oracle
 import workloads as W
+from test_dot_sensitivity import long_step
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -79,3 +81,28 @@ def test_what_is_out_of_range_is_refused(name, p, q):
     assert (y is None) == (z is None)
     if y is not None:
         assert np.max(np.abs(y - run(name, 0, 0, 0))) < TOL
+
+
+@pytest.mark.parametrize("L,nu,nd,M", [(5, 2, 2, 40), (6, 3, 3, 50), (6, 3, 3, 60)])
+@pytest.mark.parametrize("q", [-40, -45, -63, -110])
+@pytest.mark.parametrize("schedule", [0, 2])
+def test_small_hamiltonian_is_still_orthogonalised(L, nu, nd, M, q, schedule):
+    """Gram-Schmidt terms are 1e-16 of the Hamiltonian, so in FP32 they vanish
+    first.  Steps so long that all M vectors count, and in which the basis
+    loses orthogonality without those terms (the result then moves by 1e-5,
+    1e-7 and 1e-4 of the vector).  Tolerance 1e-11 as for one pass in
+    test_gpu_exact_dots: the same space, bases that differ by roundings."""
+    m = W.random_model(L, nu, nd, seed=3, complex_hopping=True)
+    if L == 6:
+        r = np.random.default_rng(6)
+        m = W.siam_star(-1.5, 3.0, r.uniform(-3, 3, 5), r.uniform(0.2, 1.0, 5), nu, nd)
+    x = W.random_state(W.sector_dim(L, nu, nd), 20)
+    tau = long_step(oracle.Sector(m), x, M)
+    y = []
+    for s in (0, q):
+        xd = torch.from_numpy(x.copy()).cuda()
+        scaled = dict(m, **{k: np.asarray(m[k]) * 2.0 ** s for k in ("h", "eps", "U")})
+        kg.Sector(scaled).propagate(xd, tau * 2.0 ** -s, 1, kg.kg_opts_default(M=M, schedule=schedule))
+        torch.cuda.synchronize()
+        y.append(xd.cpu().numpy())
+    assert np.max(np.abs(y[1] - y[0])) < 1e-11
