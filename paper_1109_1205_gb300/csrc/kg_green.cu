@@ -463,8 +463,10 @@ int green_equilibrium_batched(kg_sector* const* s, int n_inst, const int* orb, i
 // (the multiply-add pipe is what bounds this kernel, so idle warps cost
 // nothing).  The vectors are split over gridDim.y slabs, at least eight staged
 // steps each.  48 vectors of 731,808 states: 21.8 ms in FP64 with one slab per
-// 4,096 states and whole diagonal tiles, 5 ms now; 12 vectors 1.05 -> 0.55 ms;
-// 10 vectors of 3,920 states 4.0 -> 0.06 ms.
+// 4,096 states and whole diagonal tiles, 5.0 ms now; 12 vectors 1.05 -> 0.95 ms
+// (0.55 ms when what the images leave off was dropped: 21 threads of a block have
+// outputs there, and their chains are what takes the time); 10 vectors of 3,920
+// states 4.0 -> 0.07 ms.
 constexpr int kGT = 32, kGK = 16, kGramFlush = 256;
 
 // Largest exponent field of each vector (emax pre-set to 0).
